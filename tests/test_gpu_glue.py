@@ -89,3 +89,31 @@ def test_rope(abi, L, heads, extra, dt):
         norm[:, h * 128 + 64:(h + 1) * 128] = n
     assert np.all(np.abs(got - ref) <= _half_ulp(ref, dt) + 1e-5 * norm)
     assert np.array_equal(got[:, heads * 128:], x[:, heads * 128:])
+
+
+# one item per thread at most (1, 3 heads), several per thread (33, 64 heads);
+# rows off a 16-byte boundary (odd ld, or a view starting 2 bytes in) take the
+# element-wise form
+@pytest.mark.parametrize("L,heads,extra,off,dt", [(1, 1, 0, 0, "bf16"), (7, 3, 8, 0, "f16"), (3, 64, 0, 0, "f16"),
+                                                  (5, 33, 128, 0, "bf16"), (4, 33, 7, 0, "bf16"), (4, 2, 8, 1, "f16")])
+def test_rope_items_and_alignment(abi, L, heads, extra, off, dt):
+    rng = np.random.default_rng(L * heads + extra + off)
+    C = heads * 128 + extra
+    x = _round(rng.normal(0, 1, (L, C)).astype(np.float32), dt)
+    pos = rng.integers(0, 8192, L).astype(np.int32)
+    QK = H.dev(x, H.torch_dtype(dt))
+    view = QK[:, off:]
+    abi.rope(view, heads if not off else heads - 1, H.dev(pos), 1e4)
+    torch.cuda.synchronize()
+    nh = heads if not off else heads - 1
+    ang = pos.astype(np.float32)[:, None] * og.rope_frequencies(1e4).astype(np.float32)[None, :]
+    xv = x[:, off:]
+    ref = og.rope(xv, pos, nh, 1e4, angles=ang)
+    got = H.host(QK).astype(np.float64)[:, off:]
+    pair = np.stack([xv[:, h * 128 + i:h * 128 + i + 64] for h in range(nh) for i in (0, 64)], 1).astype(np.float64)
+    n = np.sqrt(pair[:, 0::2] ** 2 + pair[:, 1::2] ** 2)
+    norm = np.zeros_like(ref)
+    norm[:, : nh * 128] = np.concatenate([n, n], 2).reshape(L, -1)
+    assert np.all(np.abs(got - ref) <= _half_ulp(ref, dt) + 1e-5 * norm)
+    assert np.array_equal(got[:, nh * 128:], xv[:, nh * 128:])
+    assert np.array_equal(H.host(QK)[:, :off], x[:, :off])
