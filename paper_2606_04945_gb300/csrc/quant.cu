@@ -408,64 +408,81 @@ template <> struct To<float> { static __device__ __forceinline__ float f(float h
 
 // ---------------------------------------------------------------------------
 // Rows with Hadamard blocks of 1024 elements or more (hb >= 1024, K a
-// multiple of 1024, K <= 4096 NR), or of at most 512 (1024 <= K <= 4096,
-// K % 512 == 0, a last chunk of 512 allowed): one CTA of four warps per
-// row, in rounds of 4096 elements (four 1024-element chunks, chunk j of a
-// round in warp j).
-// A warp reads its chunk of x and of the smoothing vector with coalesced
-// 16-byte loads (lane l at 16 l + 512 q) and passes each through its
-// shared slice to take it back in layout A (18 KB of shared memory per CTA,
-// so registers, not shared memory, bound the CTAs per SM).
+// multiple of 1024), or of at most 512 (K >= 1024, K % 512 == 0, a last chunk
+// of 512 allowed): one CTA of four warps per 4096-element slice of a row, a
+// 1024-element chunk per warp (element e of the chunk: bits 0 .. 9). Each
+// layout keeps five element bits in a thread's 32 registers, so that the
+// stages over those bits are between registers:
 //
-//   layout A  lane l holds elements 32 l .. 32 l + 31 of its warp's chunk:
-//             stages h = 1 .. 16 are between registers;
-//   layout B  lane l holds elements l + 32 i (i = 0 .. 31) of the chunk,
-//             after a transpose through the chunk's shared slice: stages
-//             h = 32 .. 512 are between registers;
-//   layout C  after the round's four chunks are in shared memory, lane l of
-//             warp w holds elements j 1024 + 256 w + 8 l .. + 7 of every
-//             chunk j: stages h = 1024, 2048 are between registers, and the
-//             eight consecutive codes per chunk pack into one 32-bit word.
+//   layout 1  bits 0, 1, 7, 8, 9 (register 4 q + k: element 4 l + 128 q + k of
+//             lane l): the layout of the loads -- x and the smoothing vector
+//             meet as they arrive, 8 or 16 bytes per lane -- and of the codes.
+//             Stages h = 1, 2, and after layout 2 h = 128, 256, 512;
+//   layout 2  bits 2 .. 6 (register i: element (l & 3) + 4 i + 128 (l >> 2)):
+//             stages h = 4 .. 64;
+//   layout 3  hb > 1024 only: bits 0, 1, 7 and the chunk number (register
+//             8 j + 4 q + k: element 256 w + 128 q + 4 l + k of chunk j for
+//             lane l of warp w): stages h = 1024, 2048.
+//
+// The layouts change through the warp's own slice of shared memory, eight
+// rows (q) of 128 floats padded to 132: the 16-byte accesses of layouts 1 and
+// 3 and the 4-byte accesses of layout 2 are all free of bank conflicts, and
+// every address is a per-thread base plus a constant. Only layout 3 and the
+// row maximum need the whole CTA.
+//
+// Bound by instruction issue (67% of the slots at 8192 x 4096) and shared-
+// memory wavefronts (74%), not by HBM. An earlier split (32 consecutive
+// elements per lane first, then two more layouts) staged x and the smoothing
+// vector through shared memory to reach its first layout: 224 wavefronts per
+// 1024 elements instead of 128 (192 with layout 3), and 1141 warp instructions
+// instead of 859 (1349 for the present split with the Hadamard block known
+// only at run time: the branches around the stages keep the register pairs
+// apart). Microseconds back to back, before and now: 8192 x 4096 fp16, hb 4096
+// 43.0, 35.1; 8192 x 3584 bf16, hb 512 39.8, 29.3; 8192 x 18944 245.6, 176.2;
+// 1024 x 12288 23.5, 18.0; 1024 x 4096 8.3, 6.5; codes of 24576 x 4096 weights
+// 120.5, 97.7.
 // Butterflies on pairs of registers use the packed f32x2 add and subtract
-// (each half rounds like the scalar operation). The shared slice of a chunk
-// holds its 32 x 32 floats in rows of 36 (four floats of padding): row r
-// starts 4 r banks further on, so the row-wise 16-byte accesses (layouts A
-// and C, eight lanes per phase) and the column-wise 4-byte accesses (layout
-// B) are all free of bank conflicts, and every address is a per-thread base
-// plus a constant.
+// (each half rounds like the scalar operation).
 // ---------------------------------------------------------------------------
-constexpr int SROW = 36;                                   // floats per row of a 32 x 32 slice
-constexpr int SLICE = 32 * SROW;                           // floats per slice
-__device__ __forceinline__ int pad(int row, int col) {     // float index in a padded slice
-    return row * SROW + col;
+constexpr int MAX_SLICES = 5;                              // K <= 20480
+constexpr int QROW = 132;                                  // floats per 128-element row of a slice
+constexpr int SLICE = 8 * QROW;                            // floats per slice
+
+using f32x2 = unsigned long long;                          // two float32 in a register pair
+__device__ __forceinline__ f32x2 pack2f(float lo, float hi) {
+    f32x2 p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(lo), "f"(hi));
+    return p;
+}
+__device__ __forceinline__ void unpack2f(f32x2 p, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ void butterfly2(f32x2& a, f32x2& b) {
+    f32x2 s, d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(a), "l"(b));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    a = s;
+    b = d;
 }
 
-// Two butterflies (a0, b0) and (a1, b1) with one packed add and one packed
-// subtract: a' = a + b, b' = a - b.
-__device__ __forceinline__ void butterfly2(float& a0, float& a1, float& b0, float& b1) {
-    asm("{\n\t.reg .b64 A, B, S, D;\n\t"
-        "mov.b64 A, {%0, %1};\n\t"
-        "mov.b64 B, {%2, %3};\n\t"
-        "add.rn.f32x2 S, A, B;\n\t"
-        "sub.rn.f32x2 D, A, B;\n\t"
-        "mov.b64 {%0, %1}, S;\n\t"
-        "mov.b64 {%2, %3}, D;\n\t}"
-        : "+f"(a0), "+f"(a1), "+f"(b0), "+f"(b1));
-}
-
-// In-register stages of a 32-value array for register distances
-// s = s_lo .. s_end / 2 (s = 1 scalar, s >= 2 on packed pairs).
-__device__ __forceinline__ void reg_stages32(float (&v)[32], int s_lo, int s_end) {
+// In-register stages of 32 values (pair i: registers 2 i, 2 i + 1) for the
+// register distances s = s_lo .. s_end / 2 (s = 1 scalar, s >= 2 packed).
+__device__ __forceinline__ void reg_stages32(f32x2 (&p)[16], int s_lo, int s_end) {
     if (s_lo <= 1 && 1 < s_end) {
         #pragma unroll
-        for (int i = 0; i < 32; i += 2) butterfly(v[i], v[i + 1]);
+        for (int i = 0; i < 16; ++i) {
+            float x, y;
+            unpack2f(p[i], x, y);
+            butterfly(x, y);
+            p[i] = pack2f(x, y);
+        }
     }
     #pragma unroll
     for (int s = 2; s < 32; s <<= 1) {
         if (s >= s_lo && s < s_end) {
             #pragma unroll
-            for (int i = 0; i < 32; i += 2)
-                if ((i & s) == 0) butterfly2(v[i], v[i + 1], v[i + s], v[i + s + 1]);
+            for (int i = 0; i < 16; ++i)
+                if ((i & (s / 2)) == 0) butterfly2(p[i], p[i + s / 2]);
         }
     }
 }
@@ -490,47 +507,53 @@ __device__ __forceinline__ void quant_pair(float v0, float v1, float r, float& q
     i1 -= 0x4B400000;
 }
 
-// Eight codes (ints) -> packed nibbles, code k in bits 4k .. 4k + 3.
-__device__ __forceinline__ uint32_t pack_nibbles8(const int* qi) {
-    uint32_t w = 0;
+// Four codes (floats) -> their E4M3 bytes (byte k = code k).
+__device__ __forceinline__ uint32_t e4m3_bytes4(const float* qf) {
+    uint16_t h[2];
     #pragma unroll
-    for (int k = 6; k >= 0; k -= 2)      // d = c << 8 | sat4(a) << 4 | sat4(b)
-        asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %0;" : "+r"(w) : "r"(qi[k + 1]), "r"(qi[k]));
-    return w;
-}
-// Eight codes (floats) -> their eight E4M3 bytes (byte k = code k).
-__device__ __forceinline__ uint2 e4m3_bytes8(const float* qf) {
-    uint16_t h[4];
-    #pragma unroll
-    for (int k = 0; k < 4; ++k)          // upper byte from the first operand
+    for (int k = 0; k < 2; ++k)          // upper byte from the first operand
         asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(h[k]) : "f"(qf[2 * k + 1]), "f"(qf[2 * k]));
-    return make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16));
+    return (uint32_t)h[0] | ((uint32_t)h[1] << 16);
 }
 
-__device__ __forceinline__ float ld_shared_cluster_f32(uint32_t cluster_addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
-    return v;
+__device__ __forceinline__ void st_shared_cluster_f32(uint32_t cluster_addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" :: "r"(cluster_addr), "f"(v) : "memory");
 }
 
-// ASYM: the asymmetric mode (a compile-time copy, so that the symmetric
-// kernel carries none of its reductions). CL > 1 (with NR = 1): a cluster
-// of CL CTAs per row, CTA r taking the row's features 4096 r .. 4096 r +
-// 4095; the CTAs exchange their maxima through distributed shared memory,
-// so no thread holds more than one 4096-feature slice.
+// Four consecutive elements of a row as loaded, and as float32.
+template <typename T> struct Raw4 { using V = uint2; };
+template <> struct Raw4<float> { using V = float4; };
+template <typename T>
+__device__ __forceinline__ void raw4_to_f(const uint2& w, float* f) {
+    const T* h = reinterpret_cast<const T*>(&w);
+    #pragma unroll
+    for (int k = 0; k < 4; ++k) f[k] = To<T>::f(h[k]);
+}
+template <typename T>
+__device__ __forceinline__ void raw4_to_f(const float4& w, float* f) {
+    f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
+}
+
+// HB: the Hadamard block when it is known at compile time (no branch around
+// any stage), or 0 to take it from the arguments. ASYM: the asymmetric mode (a
+// compile-time copy, so that the symmetric kernel carries none of its
+// reductions). CLUSTER: a cluster of CTAs per row, CTA r taking the row's
+// features 4096 r .. 4096 r + 4095; the CTAs exchange their maxima through
+// distributed shared memory, so no thread holds more than one 4096-feature
+// slice.
 // G2: rows a0.L .. a0.L + b.L - 1 of the grid quantise problem b (the same
 // K, hb, input type and code width; its own X, mask, transform and outputs):
 // two quantisations in one launch.
-template <int NR, typename Tin, bool ASYM, int CL = 1, bool G2 = false>
-__global__ void __launch_bounds__(128, NR == 1 ? 7 : 1)
-sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b) {
-    static_assert(CL == 1 || NR == 1, "one slice per CTA of a cluster");
-    static_assert(!G2 || CL == 1, "grouped launches run one CTA per row");
+template <typename Tin, int HB, bool ASYM, bool CLUSTER, bool G2>
+__global__ void __launch_bounds__(128, 7)
+sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
+    static_assert(!G2 || !CLUSTER, "grouped launches run one CTA per row");
+    using Raw = typename Raw4<Tin>::V;
     const bool p1 = G2 && (int)blockIdx.x >= a0.L;
     const QuantArgs& a = p1 ? b : a0;
     __shared__ __align__(16) float buf[4 * SLICE];
     __shared__ float red[8];              // [0, 4) amax or X_max, [4, 8) -X_min (asym)
-    __shared__ float cl_red[2];           // this CTA's maximum (and -minimum) for its cluster
+    __shared__ float cl_red[2][MAX_SLICES];   // the maxima (and -minima) of the row's slices
     // launched with programmatic serialisation: the rows of a problem whose
     // caller vouches that the preceding launch neither writes its inputs
     // nor touches its outputs start without waiting for that launch
@@ -538,169 +561,125 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b) {
     grid_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int rank = CL > 1 ? (int)cluster_ctarank() : 0;
-    const int row = CL > 1 ? (int)blockIdx.x / CL : (int)blockIdx.x - (p1 ? a0.L : 0);
-    const int K = a.K;
+    const int rank = CLUSTER ? (int)cluster_ctarank() : 0;
+    const int row = CLUSTER ? (int)blockIdx.x / ctas_per_row : (int)blockIdx.x - (p1 ? a0.L : 0);
+    const int K = a.K, hb = HB > 0 ? HB : a.hb;
     const bool masked = a.mask != nullptr && a.mask[row] != 0;
     const float* sm = masked ? a.a_m : a.a_u;
-    const int own_lo = masked ? a.d_sh : a.d_sh + a.d_m;
-    const int own_hi = masked ? a.d_sh + a.d_m : K;
     const Tin* X = static_cast<const Tin*>(a.X) + (size_t)row * K;
-    float* slice = buf + warp * SLICE;
+    const int base = rank * 4096;
+    const int c0 = base + warp * 1024;                           // first element of the warp's chunk
+    const bool live = c0 < K;
+    const bool half = K - c0 < 1024;      // a last chunk of 512: its upper half is zeros, never stored
+    float* own = buf + warp * SLICE + 4 * lane;                  // layout 1: row q at own + QROW q
+    float* tr = buf + warp * SLICE + (lane & 3) + QROW * (lane >> 2);   // layout 2: register i at tr + 4 i
 
-    float v[NR][32];                      // layout C: v[R][8 j + k]
-    float amax = 0.f, nmin = 0.f;         // asym: X_max and -X_min
-    #pragma unroll
-    for (int R = 0; R < NR; ++R) {
-        const int base = (rank + R) * 4096;
-        const int nch = min(4, (K - base + 1023) >> 10); // chunks in this round (>= 1)
-        float u[32];
-        if (warp < nch) {
-            // coalesced loads (lane l: 16 bytes at 16 l + 512 q); x and then
-            // the smoothing vector pass through the warp's slice and come
-            // back in layout A
-            const int c0 = base + warp * 1024;                   // first element of the chunk
-            // a last chunk of 512 (hb <= 512 only): the upper half is zeros,
-            // its own Hadamard blocks, never stored
-            const bool half = K - c0 < 1024;
-            float4 sr[8];
-            if (sizeof(Tin) == 2) {
-                uint4 xr[4];
-                #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    xr[q] = (!half || q < 2) ? __ldg(reinterpret_cast<const uint4*>(X + c0) + lane + 32 * q)
-                                             : make_uint4(0u, 0u, 0u, 0u);
-                // 16-bit staging: 32 rows of 64 bytes, 16-byte group g of row R at g ^ ((R >> 1) & 3)
-                uint8_t* st8 = reinterpret_cast<uint8_t*>(slice);
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int R = (lane >> 2) + 8 * q, g = lane & 3;
-                    *reinterpret_cast<uint4*>(st8 + R * 64 + 16 * (g ^ ((R >> 1) & 3))) = xr[q];
-                }
-                if (sm != nullptr) {
-                    #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        sr[q] = (!half || q < 4) ? __ldg(reinterpret_cast<const float4*>(sm + c0) + lane + 32 * q)
-                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                __syncwarp();
-                #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const uint4 w = *reinterpret_cast<const uint4*>(st8 + lane * 64 + 16 * (g ^ ((lane >> 1) & 3)));
-                    const Tin* h = reinterpret_cast<const Tin*>(&w);
-                    #pragma unroll
-                    for (int k = 0; k < 8; ++k) u[8 * g + k] = To<Tin>::f(h[k]);
-                }
-            } else {
-                float4 xr[8];
-                #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    xr[q] = (!half || q < 4) ? __ldg(reinterpret_cast<const float4*>(X + c0) + lane + 32 * q)
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
-                #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<float4*>(slice + pad((lane >> 3) + 4 * q, 4 * (lane & 7))) = xr[q];
-                if (sm != nullptr) {
-                    #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        sr[q] = (!half || q < 4) ? __ldg(reinterpret_cast<const float4*>(sm + c0) + lane + 32 * q)
-                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                __syncwarp();
-                #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 w = *reinterpret_cast<const float4*>(slice + pad(lane, 4 * q));
-                    u[4 * q] = w.x; u[4 * q + 1] = w.y; u[4 * q + 2] = w.z; u[4 * q + 3] = w.w;
-                }
-            }
-            if (sm != nullptr) {
-                __syncwarp();                                    // x has left the slice
-                #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<float4*>(slice + pad((lane >> 3) + 4 * q, 4 * (lane & 7))) = sr[q];
-                __syncwarp();
-                #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 w = *reinterpret_cast<const float4*>(slice + pad(lane, 4 * q));
-                    u[4 * q] = __fmul_rn(u[4 * q], w.x);
-                    u[4 * q + 1] = __fmul_rn(u[4 * q + 1], w.y);
-                    u[4 * q + 2] = __fmul_rn(u[4 * q + 2], w.z);
-                    u[4 * q + 3] = __fmul_rn(u[4 * q + 3], w.w);
-                }
-            }
-            __syncwarp();
-            reg_stages32(u, 1, a.hb < 32 ? a.hb : 32);          // h = 1 .. min(hb, 32) / 2
-            #pragma unroll
-            for (int q = 0; q < 8; ++q)                          // layout A -> slice
-                *reinterpret_cast<float4*>(slice + pad(lane, 4 * q)) =
-                    make_float4(u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
-            __syncwarp();
-            #pragma unroll
-            for (int i = 0; i < 32; ++i) u[i] = slice[pad(i, lane)];   // layout B
-            reg_stages32(u, 1, a.hb / 32);                       // h = 32 .. min(hb, 1024) / 2
-            #pragma unroll
-            for (int i = 0; i < 32; ++i) slice[pad(i, lane)] = u[i];
+    f32x2 p[16];
+    auto put_own = [&]() {                                       // layout 1 -> the warp's slice
+        #pragma unroll
+        for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<ulonglong2*>(own + QROW * q) = make_ulonglong2(p[2 * q], p[2 * q + 1]);
+    };
+    if (live) {
+        Raw xr[8];
+        float4 sr[8];
+        const Raw* x4 = reinterpret_cast<const Raw*>(X + c0) + lane;
+        #pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            xr[q] = Raw();
+            if (!half || q < 4) xr[q] = __ldg(x4 + 32 * q);
         }
+        if (sm != nullptr) {
+            const float4* s4 = reinterpret_cast<const float4*>(sm + c0) + lane;
+            #pragma unroll
+            for (int q = 0; q < 8; ++q)
+                sr[q] = (!half || q < 4) ? __ldg(s4 + 32 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+            #pragma unroll
+            for (int q = 0; q < 8; ++q) sr[q] = make_float4(1.f, 1.f, 1.f, 1.f);   // x * 1 = x
+        }
+        #pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            float f[4];
+            raw4_to_f<Tin>(xr[q], f);
+            p[2 * q] = pack2f(__fmul_rn(f[0], sr[q].x), __fmul_rn(f[1], sr[q].y));
+            p[2 * q + 1] = pack2f(__fmul_rn(f[2], sr[q].z), __fmul_rn(f[3], sr[q].w));
+        }
+        reg_stages32(p, 1, hb < 4 ? hb : 4);                     // h = 1, 2
+        if (hb > 4) {
+            put_own();                                           // layout 1 -> 2
+            __syncwarp();
+            #pragma unroll
+            for (int i = 0; i < 16; ++i) p[i] = pack2f(tr[8 * i], tr[8 * i + 4]);
+            reg_stages32(p, 1, hb / 4);                          // h = 4 .. min(hb, 128) / 2
+            #pragma unroll
+            for (int i = 0; i < 16; ++i) unpack2f(p[i], tr[8 * i], tr[8 * i + 4]);   // layout 2 -> 1
+            __syncwarp();
+            #pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(own + QROW * q);
+                p[2 * q] = w.x;
+                p[2 * q + 1] = w.y;
+            }
+            reg_stages32(p, 4, hb / 32);                         // h = 128 .. min(hb, 1024) / 2
+        }
+    } else {
+        #pragma unroll
+        for (int i = 0; i < 16; ++i) p[i] = 0;
+    }
+    // group g of four registers: elements e_base + (g >> 1) e_step + 128 (g & 1) ..
+    int e_base = c0 + 4 * lane, e_step = 256;
+    if (hb > 1024) {                                             // layout 1 -> 3
+        e_base = base + warp * 256 + 4 * lane;
+        e_step = 1024;
+        if (live) put_own();
         __syncthreads();
         #pragma unroll
-        for (int j = 0; j < 4; ++j) {                            // layout C
-            if (j < nch) {
-                const int r = warp * 8 + (lane >> 2), c = (lane & 3) * 8;
-                const float4 p0 = *reinterpret_cast<const float4*>(buf + j * SLICE + pad(r, c));
-                const float4 p1 = *reinterpret_cast<const float4*>(buf + j * SLICE + pad(r, c + 4));
-                v[R][8 * j] = p0.x; v[R][8 * j + 1] = p0.y; v[R][8 * j + 2] = p0.z; v[R][8 * j + 3] = p0.w;
-                v[R][8 * j + 4] = p1.x; v[R][8 * j + 5] = p1.y; v[R][8 * j + 6] = p1.z; v[R][8 * j + 7] = p1.w;
-            } else {
-                #pragma unroll
-                for (int k = 0; k < 8; ++k) v[R][8 * j + k] = 0.f;
-            }
+        for (int g = 0; g < 8; ++g) {
+            ulonglong2 w = make_ulonglong2(0, 0);
+            if (base + (g >> 1) * 1024 < K)                      // chunk g >> 1 exists
+                w = *reinterpret_cast<const ulonglong2*>(buf + (g >> 1) * SLICE + QROW * (2 * warp + (g & 1)) +
+                                                         4 * lane);
+            p[2 * g] = w.x;
+            p[2 * g + 1] = w.y;
         }
-        if (NR > 1) __syncthreads();                             // the next round reuses buf
-        if (a.hb > 1024) {                                       // h = 1024: chunks j, j ^ 1
-            #pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                butterfly2(v[R][k], v[R][k + 1], v[R][8 + k], v[R][9 + k]);
-                butterfly2(v[R][16 + k], v[R][17 + k], v[R][24 + k], v[R][25 + k]);
-            }
-        }
-        if (a.hb > 2048) {                                       // h = 2048: chunks j, j ^ 2
-            #pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                butterfly2(v[R][k], v[R][k + 1], v[R][16 + k], v[R][17 + k]);
-                butterfly2(v[R][8 + k], v[R][9 + k], v[R][24 + k], v[R][25 + k]);
-            }
-        }
+        reg_stages32(p, 8, hb / 128);                            // h = 1024, 2048
+    }
+    auto first = [&](int g) { return e_base + (g >> 1) * e_step + (g & 1) * 128; };   // element of group g
+    float v[32];
+    #pragma unroll
+    for (int i = 0; i < 16; ++i) unpack2f(p[i], v[2 * i], v[2 * i + 1]);
+    if (first(7) + 4 > a.d_sh) {          // the lane reaches past the shared coordinates: the gate
+        const int own_lo = masked ? a.d_sh : a.d_sh + a.d_m;
+        const int own_hi = masked ? a.d_sh + a.d_m : K;
         #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int e0 = base + j * 1024 + warp * 256 + 8 * lane;    // first element of the group
-            if (j >= nch || e0 >= K) continue;
-            const bool all_keep = (e0 + 8 <= a.d_sh) || (e0 >= own_lo && e0 + 8 <= own_hi);
-            if (!all_keep) {
-                #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int e = e0 + k;
-                    if (!(e < a.d_sh || (e >= own_lo && e < own_hi))) v[R][8 * j + k] = 0.f;
-                }
-            }
-            if (a.post_scale != 1.f) {
-                #pragma unroll
-                for (int k = 0; k < 8; ++k) v[R][8 * j + k] = __fmul_rn(v[R][8 * j + k], a.post_scale);
-            }
-            if (ASYM) {
-                #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    amax = fmaxf(amax, v[R][8 * j + k]);
-                    nmin = fmaxf(nmin, -v[R][8 * j + k]);
-                }
-            } else {
-                #pragma unroll
-                for (int k = 0; k < 8; ++k) amax = fmaxf(amax, fabsf(v[R][8 * j + k]));
-            }
-            if (a.v_dbg != nullptr) {
-                float4* d4 = reinterpret_cast<float4*>(a.v_dbg + (size_t)row * K + e0);
-                d4[0] = make_float4(v[R][8 * j], v[R][8 * j + 1], v[R][8 * j + 2], v[R][8 * j + 3]);
-                d4[1] = make_float4(v[R][8 * j + 4], v[R][8 * j + 5], v[R][8 * j + 6], v[R][8 * j + 7]);
-            }
+        for (int g = 0; g < 8; ++g) {
+            const int e0 = first(g);
+            #pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (e0 + k >= a.d_sh && (e0 + k < own_lo || e0 + k >= own_hi)) v[4 * g + k] = 0.f;
+        }
+    }
+    if (a.post_scale != 1.f) {
+        #pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = __fmul_rn(v[i], a.post_scale);
+    }
+    if (a.v_dbg != nullptr) {
+        #pragma unroll
+        for (int g = 0; g < 8; ++g)
+            if (first(g) < K)
+                *reinterpret_cast<float4*>(a.v_dbg + (size_t)row * K + first(g)) =
+                    make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+    }
+    // (values past the row's end are zeros)
+    float amax = 0.f, nmin = 0.f;         // asym: X_max and -X_min
+    #pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        if (ASYM) {
+            amax = fmaxf(amax, v[i]);
+            nmin = fmaxf(nmin, -v[i]);
+        } else {
+            amax = fmaxf(amax, fabsf(v[i]));
         }
     }
     #pragma unroll
@@ -716,16 +695,18 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b) {
     __syncthreads();
     amax = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
     if (ASYM) nmin = fmaxf(fmaxf(red[4], red[5]), fmaxf(red[6], red[7]));
-    if (CL > 1) {                      // the row's maximum over the cluster's slices
-        if (threadIdx.x == 0) {
-            cl_red[0] = amax;
-            cl_red[1] = nmin;
+    if (CLUSTER) {
+        // the row's maximum over the cluster's slices: every CTA writes its
+        // own into all of them, so that after the one barrier nobody reads
+        // another CTA's memory and each may finish by itself
+        if ((int)threadIdx.x < ctas_per_row) {
+            st_shared_cluster_f32(mapa_shared(smem_addr(&cl_red[0][rank]), threadIdx.x), amax);
+            if (ASYM) st_shared_cluster_f32(mapa_shared(smem_addr(&cl_red[1][rank]), threadIdx.x), nmin);
         }
         cluster_sync();
-        #pragma unroll
-        for (int c = 0; c < CL; ++c) {
-            amax = fmaxf(amax, ld_shared_cluster_f32(mapa_shared(smem_addr(&cl_red[0]), (uint32_t)c)));
-            if (ASYM) nmin = fmaxf(nmin, ld_shared_cluster_f32(mapa_shared(smem_addr(&cl_red[1]), (uint32_t)c)));
+        for (int c = 0; c < ctas_per_row; ++c) {
+            amax = fmaxf(amax, cl_red[0][c]);
+            if (ASYM) nmin = fmaxf(nmin, cl_red[1][c]);
         }
     }
 
@@ -741,100 +722,98 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b) {
     }
     if (ASYM && a.Xe != nullptr && threadIdx.x < 8 && rank == 0)
         store_zero_point_columns(a.Xe + (size_t)row * (K + 128) + K, zp, threadIdx.x);
-    #pragma unroll
-    for (int R = 0; R < NR; ++R) {
-        const int base = (rank + R) * 4096;
-        const int nch = min(4, (K - base + 1023) >> 10);
-        #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int e0 = base + j * 1024 + warp * 256 + 8 * lane;
-            if (j >= nch || e0 >= K) continue;
-            float qf[8];
-            int qi[8];
+    // codes of group g, as integers and as floats
+    auto codes = [&](int g, float (&qf)[4], int (&qi)[4]) {
+        quant_pair(v[4 * g], v[4 * g + 1], r, qf[0], qf[1], qi[0], qi[1]);
+        quant_pair(v[4 * g + 2], v[4 * g + 3], r, qf[2], qf[3], qi[2], qi[3]);
+        if (ASYM) {
             #pragma unroll
-            for (int k = 0; k < 8; k += 2)
-                quant_pair(v[R][8 * j + k], v[R][8 * j + k + 1], r, qf[k], qf[k + 1], qi[k], qi[k + 1]);
-            if (ASYM) {                  // codes in [0, qmax]: unsigned nibbles and E4M3 bytes
-                int q[8];
-                #pragma unroll
-                for (int k = 0; k < 8; ++k) q[k] = min(max(qi[k] + zp, 0), a.qmax);
-                if (a.Xq != nullptr) *reinterpret_cast<uint32_t*>(a.Xq + (size_t)row * (K / 2) + e0 / 2) = pack8(q);
-                if (a.Xe != nullptr) *reinterpret_cast<uint2*>(a.Xe + (size_t)row * (K + 128) + e0) = e4m3_of8(q);
-                continue;
+            for (int k = 0; k < 4; ++k) {
+                qi[k] = min(max(qi[k] + zp, 0), a.qmax);
+                qf[k] = (float)qi[k];
             }
-            if (a.qmax > 15) {           // 8-bit codes: bytes and fp16
-                uint2 bytes;
-                uint4 f16;
-                codes8(qi, bytes, f16);
-                if (a.Xq != nullptr) *reinterpret_cast<uint2*>(a.Xq + (size_t)row * K + e0) = bytes;
-                if (a.Xe != nullptr) *reinterpret_cast<uint4*>(a.Xe + ((size_t)row * K + e0) * 2) = f16;
-                continue;
-            }
-            if (a.Xq != nullptr)
-                *reinterpret_cast<uint32_t*>(a.Xq + (size_t)row * (K / 2) + e0 / 2) = pack_nibbles8(qi);
-            if (a.Xe != nullptr) *reinterpret_cast<uint2*>(a.Xe + (size_t)row * K + e0) = e4m3_bytes8(qf);
+        }
+    };
+    const bool wide = !ASYM && a.qmax > 15;                      // 8-bit codes: fp16 and bytes
+    if (a.Xe != nullptr && wide) {
+        uint8_t* dst = a.Xe + (size_t)row * K * 2;
+        #pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            float qf[4];
+            int qi[4];
+            codes(g, qf, qi);
+            const __half2 h0 = __floats2half2_rn(qf[0], qf[1]), h1 = __floats2half2_rn(qf[2], qf[3]);
+            if (first(g) < K)
+                *reinterpret_cast<uint2*>(dst + 2 * first(g)) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+        }
+    } else if (a.Xe != nullptr) {                                // E4M3 bytes
+        uint8_t* dst = a.Xe + (size_t)row * (ASYM ? K + 128 : K);
+        #pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            float qf[4];
+            int qi[4];
+            codes(g, qf, qi);
+            if (first(g) < K) *reinterpret_cast<uint32_t*>(dst + first(g)) = e4m3_bytes4(qf);
         }
     }
-    if (CL > 1) cluster_sync();        // no CTA leaves while its maximum may still be read
+    if (a.Xq != nullptr) {
+        uint8_t* dst = a.Xq + (size_t)row * (wide ? K : K / 2);
+        #pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            float qf[4];
+            int qi[4];
+            codes(g, qf, qi);
+            if (first(g) >= K) continue;
+            if (wide)
+                *reinterpret_cast<uint32_t*>(dst + first(g)) =
+                    prmt(prmt((uint32_t)qi[0], (uint32_t)qi[1], 0x0040u),
+                         prmt((uint32_t)qi[2], (uint32_t)qi[3], 0x0040u), 0x5410u);
+            else                         // (unsigned codes up to 15 when ASYM)
+                *reinterpret_cast<uint16_t*>(dst + first(g) / 2) =
+                    (uint16_t)((qi[0] & 15) | (qi[1] & 15) << 4 | (qi[2] & 15) << 8 | (qi[3] & 15) << 12);
+        }
+    }
 }
 
-template <int NR, typename Tin>
-cudaError_t launch_rows_nr(const QuantArgs& a, cudaStream_t stream) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1] = {pdl_attribute()};
-    cfg.gridDim = dim3(a.L);
-    cfg.blockDim = dim3(128);
-    cfg.stream = stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return a.asym ? cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<NR, Tin, true>, a, a)
-                  : cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<NR, Tin, false>, a, a);
-}
-
-// Rows longer than 4096: a cluster of CL CTAs per row, one 4096-feature
-// slice each.
-template <int CL, typename Tin>
-cudaError_t launch_rows_cl(const QuantArgs& a, cudaStream_t stream) {
+// One launch of the row kernel: a CTA per row (b != nullptr: the rows of b
+// after those of a), or beyond 4096 features a cluster of CTAs per row, one
+// 4096-feature slice each. The blocks of the model widths (512 of 3584 and
+// 18944, 4096 of 4096 and 12288) are compiled in.
+template <typename Tin, bool ASYM, bool CLUSTER, bool G2>
+cudaError_t launch_rows_kind(const QuantArgs& a, const QuantArgs& b, cudaStream_t stream) {
+    const int ctas = (a.K + 4095) / 4096;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
     at[0] = pdl_attribute();
     at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = CL;
+    at[1].val.clusterDim.x = ctas;
     at[1].val.clusterDim.y = 1;
     at[1].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)a.L * CL);
+    cfg.gridDim = dim3(CLUSTER ? (unsigned)a.L * ctas : (unsigned)(a.L + (G2 ? b.L : 0)));
     cfg.blockDim = dim3(128);
     cfg.stream = stream;
     cfg.attrs = at;
-    cfg.numAttrs = 2;
-    return a.asym ? cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<1, Tin, true, CL>, a, a)
-                  : cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<1, Tin, false, CL>, a, a);
+    cfg.numAttrs = CLUSTER ? 2 : 1;
+    if constexpr (!ASYM) {
+        if (a.hb == 4096) return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2>, a, b, ctas);
+        if (a.hb == 512) return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 512, ASYM, CLUSTER, G2>, a, b, ctas);
+    }
+    return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 0, ASYM, CLUSTER, G2>, a, b, ctas);
 }
 
-// Two symmetric quantisations of rows up to 4096 features in one launch
-// (one CTA per row of either problem).
 template <typename Tin>
 cudaError_t launch_rows_grouped(const QuantArgs& a, const QuantArgs& b, cudaStream_t stream) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1] = {pdl_attribute()};
-    cfg.gridDim = dim3((unsigned)(a.L + b.L));
-    cfg.blockDim = dim3(128);
-    cfg.stream = stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<1, Tin, false, 1, true>, a, b);
+    return launch_rows_kind<Tin, false, false, true>(a, b, stream);
 }
 
 template <typename Tin>
 cudaError_t launch_rows(const QuantArgs& a, cudaStream_t stream) {
-    switch ((a.K + 4095) / 4096) {
-        case 1: return launch_rows_nr<1, Tin>(a, stream);
-        case 2: return launch_rows_cl<2, Tin>(a, stream);
-        case 3: return launch_rows_cl<3, Tin>(a, stream);
-        case 4: return launch_rows_cl<4, Tin>(a, stream);
-        case 5: return launch_rows_cl<5, Tin>(a, stream);
-        default: return cudaErrorInvalidValue;
-    }
+    if (a.K > 4096)
+        return a.asym ? launch_rows_kind<Tin, true, true, false>(a, a, stream)
+                      : launch_rows_kind<Tin, false, true, false>(a, a, stream);
+    return a.asym ? launch_rows_kind<Tin, true, false, false>(a, a, stream)
+                  : launch_rows_kind<Tin, false, false, false>(a, a, stream);
 }
 
 template <int E, typename Tin>
