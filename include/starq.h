@@ -459,11 +459,13 @@ int w4a4_gemm_mma_sync(const uint8_t* Xq, const float* s_a, const uint8_t* Wq, c
 /*
  * Tile of the last Xe + We (or fp16_gemm_ref) launch on the calling thread,
  * as BN * 10 + cluster size: 2562 (256-channel pair tiles) or 2242
- * (224-channel pair tiles); a cluster is one CTA pair, and each CTA loads
- * its own operand rows. 0 before the first. The launcher estimates each
- * shape's time as ceil(tiles / resident pairs) rounds of a stage cost bound
- * by shared-memory traffic and takes the cheaper. A diagnostic for tests
- * and tuning; the results do not depend on it.
+ * (224-channel pair tiles), a cluster being one CTA pair, each CTA of which
+ * loads its own operand rows; or 1281 .. 1288, the few-token kernel (128-channel
+ * tiles, K split over a cluster of 1 .. 8 CTAs). 0 before the first. The
+ * launcher estimates each shape's time (rounds of tiles over the resident
+ * pairs, the weight stream, the exchange of a split K) and takes the cheapest;
+ * under a cap on the pairs (starq_set_gemm_pair_limit) always pair tiles. A
+ * diagnostic for tests and tuning; the results do not depend on it.
  */
 int starq_last_gemm_tile(void);
 

@@ -383,8 +383,10 @@ def set_gemm_pair_limit(pairs):
 
 
 def last_gemm_tile():
-    """(channels per pair tile, CTAs per cluster) of the calling thread's
-    last TMA pair GEMM launch, or None before the first."""
+    """(channels per tile, CTAs per cluster) of the calling thread's last
+    GEMM launch on E4M3 (or 16-bit) operands, or None before the first:
+    pair tiles of 256 or 224 channels on 2 CTAs, or the few-token kernel's
+    128 channels on 1 .. 8."""
     t = int(lib.starq_last_gemm_tile())
     return (t // 10, t % 10) if t else None
 

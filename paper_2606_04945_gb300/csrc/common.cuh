@@ -73,6 +73,10 @@ struct GemmArgs {
     int swiglu = 0;
 };
 cudaError_t launch_w4a4_gemm(const GemmArgs& a, cudaStream_t stream);
+// The same product with Xe and We for few tokens (few_tokens(a)): K split over
+// a cluster of *split CTAs per 128-channel tile.
+bool few_tokens(const GemmArgs& a);
+cudaError_t launch_w4a4_gemm_few(const GemmArgs& a, int* split, cudaStream_t stream);
 // Two independent products in one persistent TMA pair launch (the same L,
 // K and output type; Xe and We given for both; no SwiGLU).
 cudaError_t launch_w4a4_gemm_grouped(const GemmArgs& a, const GemmArgs& b, cudaStream_t stream);

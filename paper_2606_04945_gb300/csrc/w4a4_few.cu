@@ -1,0 +1,376 @@
+// W4A4 GEMM for few tokens (one block of a semi-autoregressive decode, the
+// tail of a batch): the same product and dequantisation as w4a4_gemm.cu,
+//   acc[i][n] = sum_k qa[i][k] qw[n][k]        exact integer sums in float32
+//   Y[i][n]   = fl(fl(acc * s_a[i]) * s_w[n]) (+ bias[n]) -> output type
+// with E4M3 operands, organised around the weight stream.
+//
+// With few tokens the floor is reading the weights' N K bytes from HBM once,
+// and what matters is how many of them are in flight on how many SMs. The
+// 256-token pair tiles of w4a4_gemm.cu give ceil(N / 224) pairs, each walking
+// the whole K chain alone: 110 of 152 SMs at N = 12288, 38 at N = 4096. Here
+// the operands trade places: 128 weight rows are the M of the MMA and the
+// tokens (16, 32, 64 or 128 rows) its N, one CTA per (128-channel tile, part of
+// K), two CTAs per SM with ~100 KB of tiles in flight each. The S parts of K of
+// one tile are a cluster: every CTA sends its partial sums (integers, exact in
+// float32, so their order does not matter) of token t to part t mod S through
+// distributed shared memory, a 128-byte line per warp and token, and each
+// part adds up and dequantises its own tokens. (Reading the other parts' sums
+// instead, 16-byte remote stores by token groups, and bulk copies between the
+// shared memories were 1 to 6 us slower at 64 tokens.)
+//
+//   warp 4    TMA: weight and token tiles of 128 K through a ring of stages
+//             (the weights of the first stages ahead of the wait for the
+//             previous kernel when the caller vouches for them);
+//   warp 5    TMEM allocation, MMA issue (tcgen05 kind::f8f6f4, M 128, N NT);
+//   warps 0-3 accumulator to the parts that own the tokens, their sums,
+//             dequantisation, stores.
+// Every wait is bounded; a CTA that gives up records it in the status word
+// and still takes part in the cluster barriers.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include "common.cuh"
+
+namespace starq {
+namespace {
+
+namespace fewk {
+constexpr int BM = 128, BK = 128, UMMA_K = 32;           // weight rows per tile, K bytes per stage
+constexpr int A_BYTES = BM * BK;
+constexpr int NUM_EPI_WARPS = 4, TMA_WARP = 4, MMA_WARP = 5;
+constexpr int THREADS = 6 * 32;
+constexpr int MAX_SPLIT = 8;                             // portable cluster size
+template <int NT>
+struct Tile {
+    static_assert(NT % 16 == 0 && NT >= 16 && NT <= 128, "tokens per tile (MMA N)");
+    static constexpr int STAGE_BYTES = A_BYTES + NT * BK;
+    // the sums, over the stages once they are read: split * ceil(NT / split) rows of 128 channels
+    static constexpr int PART_BYTES = (NT + MAX_SPLIT - 1) * BM * 4;
+    static constexpr int FIXED = 1024 + 256;             // alignment, barriers
+    // two CTAs per SM: 113.5 KB each (227 KB less 1 KB per CTA of the system's)
+    static constexpr int STAGES = (112 * 1024 - FIXED) / STAGE_BYTES;
+    static constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + FIXED;
+    static_assert(PART_BYTES <= STAGES * STAGE_BYTES, "partial sums fit the stages");
+    static constexpr int TMEM_COLS = NT < 32 ? 32 : NT;
+    static constexpr uint32_t IDESC = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+};
+template <int S>
+struct Smem {
+    uint64_t full[S], empty[S], done;
+    uint32_t tmem_base;
+    int abort;
+};
+}  // namespace fewk
+
+template <typename T2, typename Cvt>
+__device__ __forceinline__ uint2 pack4(const float (&y)[4], Cvt cvt) {
+    const T2 a = cvt(y[0], y[1]), b = cvt(y[2], y[3]);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+__device__ __forceinline__ void store4(__half* p, const float (&y)[4]) {
+    *reinterpret_cast<uint2*>(p) = pack4<__half2>(y, [](float a, float b) { return __floats2half2_rn(a, b); });
+}
+__device__ __forceinline__ void store4(__nv_bfloat16* p, const float (&y)[4]) {
+    *reinterpret_cast<uint2*>(p) = pack4<__nv_bfloat162>(y, [](float a, float b) { return __floats2bfloat162_rn(a, b); });
+}
+__device__ __forceinline__ void store4(float* p, const float (&y)[4]) {
+    *reinterpret_cast<float4*>(p) = make_float4(y[0], y[1], y[2], y[3]);
+}
+__device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared.b32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_shared_cluster_b32(uint32_t cluster_addr, uint32_t v) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" :: "r"(cluster_addr), "r"(v) : "memory");
+}
+
+// blockIdx.x = channel tile * split + part, the cluster being the parts of one
+// tile; blockIdx.y = token tile.
+template <typename TOut, int NT>
+__global__ void __launch_bounds__(fewk::THREADS)
+w4a4_gemm_few_kernel(GemmArgs a, const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
+                     int split) {
+    using Tile = fewk::Tile<NT>;
+    constexpr int STAGES = Tile::STAGES, STAGE_BYTES = Tile::STAGE_BYTES, A_BYTES = fewk::A_BYTES, BK = fewk::BK;
+    using Smem = fewk::Smem<STAGES>;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_addr(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    Smem* sh = reinterpret_cast<Smem*>(smem_raw + (base - raw) + STAGES * STAGE_BYTES);
+    volatile int* abort = &sh->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int part = (int)cluster_ctarank();
+    const int n0 = ((int)blockIdx.x / split) * fewk::BM, n = n0 + 4 * lane;   // n: epilogue, four channels per lane
+    const int t0 = (int)blockIdx.y * NT;                     // first token of the tile
+    const int L = min(a.L - t0, NT);                         // tokens of the tile
+    const int num_k = a.K / BK;
+    const int k0 = num_k * part / split, nk = num_k * (part + 1) / split - k0;   // this part's K blocks (>= 1)
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(smem_addr(&sh->full[s]), 1);
+            mbar_init(smem_addr(&sh->empty[s]), 1);
+        }
+        mbar_init(smem_addr(&sh->done), 1);
+        sh->abort = 0;
+        mbar_fence_init();
+    }
+    if (warp == fewk::MMA_WARP) {
+        tmem_alloc(smem_addr(&sh->tmem_base), Tile::TMEM_COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = sh->tmem_base;
+    float sa_lane = 0.f;                                     // epilogue: scales and bias, read ahead
+    bool ok_epi = false;
+    float4 sw = make_float4(0.f, 0.f, 0.f, 0.f), bb = sw;
+
+    if (warp == fewk::TMA_WARP) {
+        bool ok = true;
+        const int pre = nk < STAGES ? nk : STAGES;           // first stages: no empty wait is due
+        if (elect_one()) {
+            for (int kc = 0; kc < pre; ++kc) mbar_arrive_expect_tx(smem_addr(&sh->full[kc]), STAGE_BYTES);
+            if (a.weights_ready)
+                for (int kc = 0; kc < pre; ++kc)
+                    tma_load_2d(base + kc * STAGE_BYTES, &tmap_w, (k0 + kc) * BK, n0, smem_addr(&sh->full[kc]));
+        }
+        __syncwarp();
+        grid_dependency_wait();
+        grid_launch_dependents();
+        if (elect_one()) {
+            for (int kc = 0; kc < pre; ++kc) {
+                const uint32_t st = base + kc * STAGE_BYTES, bar = smem_addr(&sh->full[kc]);
+                tma_load_2d(st + A_BYTES, &tmap_x, (k0 + kc) * BK, t0, bar);
+                if (!a.weights_ready) tma_load_2d(st, &tmap_w, (k0 + kc) * BK, n0, bar);
+            }
+        }
+        __syncwarp();
+        for (int kc = pre; kc < nk && ok; ++kc) {
+            const int s = kc % STAGES;
+            ok = mbar_wait_bounded_warp(smem_addr(&sh->empty[s]), (uint32_t)((kc / STAGES) & 1) ^ 1u, abort);
+            if (ok && elect_one()) {
+                const uint32_t st = base + s * STAGE_BYTES, bar = smem_addr(&sh->full[s]);
+                mbar_arrive_expect_tx(bar, STAGE_BYTES);
+                tma_load_2d(st, &tmap_w, (k0 + kc) * BK, n0, bar);
+                tma_load_2d(st + A_BYTES, &tmap_x, (k0 + kc) * BK, t0, bar);
+            }
+            __syncwarp();
+        }
+        if (!ok && lane == 0) { sh->abort = 1; atomicOr(a.status, STATUS_TIMEOUT_GEMM); }
+    } else if (warp == fewk::MMA_WARP) {
+        grid_dependency_wait();
+        grid_launch_dependents();
+        bool ok = true;
+        for (int kc = 0; kc < nk && ok; ++kc) {
+            const int s = kc % STAGES;
+            ok = mbar_wait_bounded_warp(smem_addr(&sh->full[s]), (uint32_t)((kc / STAGES) & 1), abort);
+            tc_fence_after();
+            if (ok && elect_one()) {
+                const uint64_t ad = smem_desc_sw128(base + s * STAGE_BYTES);
+                const uint64_t bd = smem_desc_sw128(base + s * STAGE_BYTES + A_BYTES);
+                #pragma unroll
+                for (int ks = 0; ks < BK / fewk::UMMA_K; ++ks)
+                    mma_f8f6f4(tmem, ad + (uint64_t)(ks * fewk::UMMA_K / 16), bd + (uint64_t)(ks * fewk::UMMA_K / 16),
+                               Tile::IDESC, (kc > 0 || ks > 0) ? 1u : 0u);
+                tc_commit(smem_addr(&sh->empty[s]));
+            }
+            __syncwarp();
+        }
+        if (elect_one()) tc_commit(smem_addr(&sh->done));     // also after a failed wait
+        __syncwarp();
+        if (!ok && lane == 0) { sh->abort = 1; atomicOr(a.status, STATUS_TIMEOUT_GEMM); }
+    } else {
+        grid_dependency_wait();
+        grid_launch_dependents();
+        // lane j: the activation scale of the j-th token this warp will finish
+        const int tj = part + split * (warp + fewk::NUM_EPI_WARPS * lane);
+        if (tj < L) sa_lane = __ldg(a.s_a + t0 + tj);
+        if (n < a.N) {
+            sw = __ldg(reinterpret_cast<const float4*>(a.s_w + n));
+            if (a.bias != nullptr) bb = __ldg(reinterpret_cast<const float4*>(a.bias + n));
+        }
+        volatile int never = 0;
+        ok_epi = mbar_wait_bounded_warp(smem_addr(&sh->done), 0, &never);
+        tc_fence_after();
+        if (!ok_epi && lane == 0) atomicOr(a.status, STATUS_TIMEOUT_GEMM);
+    }
+    __syncwarp();
+    if (split > 1) cluster_sync();   // every part has read its stages: they take the sums
+    // the accumulator (lane = channel, column = token): token t goes to part
+    // t mod split, into its row [this part][t / split] of 128 channels
+    const int slots = (NT + split - 1) / split;              // tokens per part
+    if (warp < fewk::NUM_EPI_WARPS && ok_epi) {
+        const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+        const uint32_t mine = base + (uint32_t)((part * slots * fewk::BM + warp * 32 + lane) * 4);
+        int owner = 0;
+        uint32_t row = 0;                                    // byte offset of row t / split
+        #pragma unroll 1
+        for (int c = 0; c < NT && c < L; c += 16) {
+            uint32_t r[16];
+            tmem_ld_32x32b_x16(trow + (uint32_t)c, r);
+            tmem_ld_wait();
+            if (split == 1) {                                // (the waiting MMAs are this CTA's own)
+                #pragma unroll
+                for (int t = 0; t < 16; ++t) st_shared_b32(mine + (uint32_t)((c + t) * fewk::BM * 4), r[t]);
+            } else {
+                #pragma unroll
+                for (int t = 0; t < 16; ++t) {
+                    st_shared_cluster_b32(mapa_shared(mine, (uint32_t)owner) + row, r[t]);
+                    if (++owner == split) { owner = 0; row += fewk::BM * 4; }
+                }
+            }
+        }
+        tc_fence_before();
+    }
+    __syncwarp();
+    // this part's tokens are complete; no part touches another's memory any more
+    if (split > 1) cluster_sync();
+    else __syncthreads();
+    if (warp < fewk::NUM_EPI_WARPS) {
+        TOut* Y = static_cast<TOut*>(a.Y);
+        int j = 0;                                           // tokens finished by this warp
+        for (int sl = warp; part + sl * split < L; sl += fewk::NUM_EPI_WARPS, ++j) {
+            const uint32_t src = base + (uint32_t)((sl * fewk::BM + 4 * lane) * 4);
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            #pragma unroll 4
+            for (int c = 0; c < split; ++c) {
+                const uint4 v = ld_shared_v4(src + (uint32_t)(c * slots * fewk::BM * 4));
+                acc.x += __uint_as_float(v.x); acc.y += __uint_as_float(v.y);
+                acc.z += __uint_as_float(v.z); acc.w += __uint_as_float(v.w);
+            }
+            const float sa = __shfl_sync(0xffffffffu, sa_lane, j);
+            float y[4] = {__fmul_rn(__fmul_rn(acc.x, sa), sw.x), __fmul_rn(__fmul_rn(acc.y, sa), sw.y),
+                          __fmul_rn(__fmul_rn(acc.z, sa), sw.z), __fmul_rn(__fmul_rn(acc.w, sa), sw.w)};
+            if (a.bias != nullptr) {
+                y[0] = __fadd_rn(y[0], bb.x);
+                y[1] = __fadd_rn(y[1], bb.y);
+                y[2] = __fadd_rn(y[2], bb.z);
+                y[3] = __fadd_rn(y[3], bb.w);
+            }
+            float h[4];
+            if (a.swiglu) {
+                // lanes 0-3 of every eight hold 16 gate channels, lanes 4-7 the matching up channels
+                #pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float up = __shfl_down_sync(0xffffffffu, y[k], 4);
+                    h[k] = y[k] / (1.f + expf(-y[k])) * up;
+                }
+            }
+            if (n >= a.N) continue;                          // (N % 32 == 0: eight lanes at a time)
+            const size_t t = (size_t)(t0 + part + sl * split);
+            if (a.acc_dbg != nullptr)
+                *reinterpret_cast<int4*>(a.acc_dbg + t * a.N + n) =
+                    make_int4(__float2int_rn(acc.x), __float2int_rn(acc.y), __float2int_rn(acc.z),
+                              __float2int_rn(acc.w));
+            if (!a.swiglu) store4(Y + t * a.N + n, y);
+            else if ((lane & 4) == 0) store4(Y + t * (a.N / 2) + n0 / 2 + (lane >> 3) * 16 + 4 * (lane & 3), h);
+        }
+    }
+    __syncwarp();
+    tc_fence_after();
+    if (warp == fewk::MMA_WARP) tmem_dealloc(tmem, Tile::TMEM_COLS);
+}
+
+bool encode_k_major(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+    const PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
+    if (fn == nullptr) return false;
+    const cuuint64_t dims[2] = {cols, rows};
+    const cuuint64_t strides[1] = {cols};
+    const cuuint32_t box[2] = {fewk::BK, box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Parts of K per tile: as many as keep every CTA resident at once (two per
+// SM), at most a portable cluster and the number of K blocks.
+int few_split(const GemmArgs& a, int token_tiles) {
+    int split = 2 * num_sms() / ((a.N + fewk::BM - 1) / fewk::BM * token_tiles);
+    if (split > fewk::MAX_SPLIT) split = fewk::MAX_SPLIT;
+    if (split > a.K / fewk::BK) split = a.K / fewk::BK;
+    return split < 1 ? 1 : split;
+}
+
+template <typename TOut, int NT>
+cudaError_t launch_few(const GemmArgs& a, int* split_used, cudaStream_t stream) {
+    using Tile = fewk::Tile<NT>;
+    auto kernel = w4a4_gemm_few_kernel<TOut, NT>;
+    static DeviceCache<int> attr;
+    int done = 0;
+    cudaError_t e = attr.get(&done, [&](int, int* v) {
+        *v = 1;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile::SMEM_BYTES);
+    });
+    if (e != cudaSuccess) return e;
+    const int tiles = (a.N + fewk::BM - 1) / fewk::BM, ytiles = (a.L + NT - 1) / NT, split = few_split(a, ytiles);
+    CUtensorMap tw, tx;
+    if (!encode_k_major(&tw, a.We, (uint64_t)a.N, (uint64_t)a.K, fewk::BM) ||
+        !encode_k_major(&tx, a.Xe, (uint64_t)a.L, (uint64_t)a.K, NT))
+        return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = split;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1] = pdl_attribute();
+    cfg.gridDim = dim3((unsigned)(tiles * split), (unsigned)ytiles);
+    cfg.blockDim = dim3(fewk::THREADS);
+    cfg.dynamicSmemBytes = Tile::SMEM_BYTES;
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    *split_used = split;
+    return cudaLaunchKernelEx(&cfg, kernel, a, tw, tx, split);
+}
+
+template <typename TOut>
+cudaError_t launch_few_typed(const GemmArgs& a, int* split_used, cudaStream_t stream) {
+    if (a.swiglu && sizeof(TOut) != 2) return cudaErrorInvalidValue;
+    if (a.L <= 16) return launch_few<TOut, 16>(a, split_used, stream);
+    if (a.L <= 32) return launch_few<TOut, 32>(a, split_used, stream);
+    if (a.L <= 64) return launch_few<TOut, 64>(a, split_used, stream);
+    return launch_few<TOut, 128>(a, split_used, stream);
+}
+
+}  // namespace
+
+// Whether this kernel is the faster one. Both estimates are fits to launches
+// back to back over weights larger than L2 (ns; L 1 .. 512, N 512 .. 24576, K
+// 512 .. 18944):
+//   pair kernel  a round of ceil(N / 224) ceil(L / 256) tiles per resident pair
+//                takes 245 ns per 128 K and 4 us of prologue and epilogue, and
+//                the weights stream at 4 TB/s at most;
+//   this kernel  1.5 us, the weights at 6 TB/s, 1.2 us for the exchange of the
+//                parts' sums, and per token 20 ns (32 when two CTAs share an
+//                SM, 70 when one CTA finishes all tokens of its tile), 1.4 times
+//                that with the shorter ring of 128-token tiles.
+// Measured, pair kernel and this one, us: 32 x 4096 -> 12288 13.6, 12.3; 32 x
+// 4096 -> 4096 12.1, 6.9; 32 x 12288 -> 4096 27.0, 11.7; 64 x 4096 -> 24576 24.9,
+// 23.1; 128 x 12288 -> 4096 27.3, 15.3; 1 x 512 -> 512 4.7, 2.5; and where it
+// stays off, 128 x 4096 -> 12288 13.8, 16.2; 128 x 3584 -> 4608 11.3, 12.0.
+bool few_tokens(const GemmArgs& a) {
+    if (a.L > 256) return false;
+    const long long bytes = (long long)a.N * a.K, num_k = a.K / fewk::BK;
+    const long long tiles = (long long)((a.N + 223) / 224), pairs = num_sms() / 2;    // (one row of tiles: L <= 256)
+    long long pair_ns = (tiles + pairs - 1) / pairs * (4000 + 245 * num_k);
+    if (pair_ns < bytes / 4000) pair_ns = bytes / 4000;
+    const int rows = a.L <= 128 ? 1 : 2, split = few_split(a, rows);
+    const int ctas = (a.N + fewk::BM - 1) / fewk::BM * rows * split;
+    long long token_ns = split == 1 ? 70 : ctas > num_sms() ? 32 : 20;
+    if (a.L > 64) token_ns = token_ns * 7 / 5;
+    return 1500 + bytes / 6000 + (split > 1 ? 1200 : 0) + token_ns * a.L < pair_ns;
+}
+
+cudaError_t launch_w4a4_gemm_few(const GemmArgs& a, int* split_used, cudaStream_t stream) {
+    switch (a.y_dtype) {
+        case STARQ_F16: return launch_few_typed<__half>(a, split_used, stream);
+        case STARQ_BF16: return launch_few_typed<__nv_bfloat16>(a, split_used, stream);
+        case STARQ_F32: return launch_few_typed<float>(a, split_used, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace starq

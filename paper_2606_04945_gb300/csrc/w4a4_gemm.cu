@@ -1624,6 +1624,12 @@ cudaError_t launch_w4a4_gemm_grouped(const GemmArgs& a, const GemmArgs& b, cudaS
 cudaError_t launch_w4a4_gemm(const GemmArgs& a, cudaStream_t stream) {
     if (a.L == 0) return cudaSuccess;
     if (a.Xe != nullptr && a.We != nullptr) {
+        if (g_pair_limit == 0 && few_tokens(a)) {      // (a cap on the CTA pairs asks for the pair kernel)
+            int split = 0;
+            const cudaError_t e = launch_w4a4_gemm_few(a, &split, stream);
+            if (e == cudaSuccess) g_last_tile = 128 * 10 + split;
+            return e;
+        }
         switch (a.y_dtype) {
             case STARQ_F16: return launch_tma_typed<__half>(a, stream);
             case STARQ_BF16: return launch_tma_typed<__nv_bfloat16>(a, stream);
