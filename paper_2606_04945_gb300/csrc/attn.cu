@@ -203,34 +203,50 @@ __device__ __forceinline__ void named_sync_softmax() {
     asm volatile("bar.sync 1, %0;" :: "r"(ATT_SOFTMAX_THREADS) : "memory");
 }
 
-// One CTA per 16 channels: two threads per key row, each holding 8
-// channels (16 bytes), 128 rows per sweep. Pass 1 takes the channel maxima,
-// pass 2 (from L2) the codes, transposed through shared memory in tiles of
-// 512 keys and written as 16-byte rows of Vt.
-constexpr int VQ_CH = 16, VQ_KEYS = 512;
+// V codes and channel scales. Bound by latency at these sizes (8 MB of V at
+// 1024 keys x 4096 channels), so the keys are split too: a CTA takes 64
+// channels (128-byte rows) of up to NCH chunks of 128 keys, and the CTAs of
+// one channel group are a cluster. V is read once, into registers; the CTA's
+// channel maxima go to every CTA of the cluster through distributed shared
+// memory, and after one cluster barrier each quantises its own keys, transposes
+// them through shared memory and writes 256-byte runs of Vt. (One CTA per 16
+// channels reading V twice took 9.1 us at 1024 x 4096 and, with 32 CTAs, 10.7 at
+// 2048 x 512.)
+// Thread (warp w, lane l): channels 8 (l mod 8) .. + 7 of the key pairs 4 w +
+// l / 8 and 32 more of each chunk. The pairs' codes are 32-bit words of the
+// transposed tile [channel][64 pairs], whose 16-byte groups are XOR-ed with
+// channel / 8, so that neither the writes nor the 16-byte reads share banks.
+constexpr int VQ_CH = 64, VQ_THREADS = 256, VQ_MAX_SPLIT = 8;
 
-template <typename T>
-__global__ void __launch_bounds__(256) attn_vquant_kernel(AttnArgs a) {
+template <typename T, int NCH>
+__global__ void __launch_bounds__(VQ_THREADS) attn_vquant_kernel(AttnArgs a, int split) {
     using T2 = typename std::conditional<std::is_same<T, __half>::value, __half2, __nv_bfloat162>::type;
-    __shared__ float red[8][VQ_CH];
+    __shared__ float red[VQ_THREADS / 32][VQ_CH];
+    __shared__ float cl_max[VQ_MAX_SPLIT][VQ_CH];          // the channel maxima of the cluster's CTAs
     __shared__ float rcp[VQ_CH];
-    __shared__ __align__(16) uint16_t tile[VQ_CH][VQ_KEYS + 8];
-    const int c0 = blockIdx.x * VQ_CH;
-    const int tid = threadIdx.x, hv = tid & 1, rr = tid >> 1, warp = tid >> 5, lane = tid & 31;
-    const T* col = static_cast<const T*>(a.V) + c0 + 8 * hv;
-    auto load = [&](int r) {
-        return r < a.L ? __ldg(reinterpret_cast<const uint4*>(col + (size_t)r * a.ld)) : make_uint4(0u, 0u, 0u, 0u);
-    };
+    __shared__ __align__(16) uint32_t tile[VQ_CH][ATTN_TILE / 2];
+    const int rank = (int)cluster_ctarank();
+    const int c0 = ((int)blockIdx.x / split) * VQ_CH;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cg = lane & 7, pair = 4 * warp + (lane >> 3);
+    const T* col = static_cast<const T*>(a.V) + c0 + 8 * cg;
+    const int chunk0 = rank * NCH, chunks = min(NCH, a.L / ATTN_TILE - chunk0);   // may be <= 0 in the last CTA
+    uint4 v[NCH][4];                                       // [chunk][2 u + (key of the pair)]
+    #pragma unroll
+    for (int j = 0; j < NCH; ++j)
+        #pragma unroll
+        for (int k = 0; k < 4; ++k)
+            v[j][k] = j < chunks ? __ldg(reinterpret_cast<const uint4*>(
+                                       col + (size_t)((chunk0 + j) * ATTN_TILE + 2 * (pair + 32 * (k >> 1)) + (k & 1)) * a.ld))
+                                 : make_uint4(0u, 0u, 0u, 0u);
     float m[8];
     #pragma unroll
     for (int k = 0; k < 8; ++k) m[k] = 0.f;
-    for (int r0 = 0; r0 < a.L; r0 += VQ_KEYS) {
-        uint4 v[4];
-        #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = load(r0 + rr + 128 * u);
+    #pragma unroll
+    for (int j = 0; j < NCH; ++j)
         #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const T2* p = reinterpret_cast<const T2*>(&v[u]);
+            const T2* p = reinterpret_cast<const T2*>(&v[j][u]);
             #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float2 f = to_float2(p[k]);
@@ -238,13 +254,12 @@ __global__ void __launch_bounds__(256) attn_vquant_kernel(AttnArgs a) {
                 m[2 * k + 1] = fmaxf(m[2 * k + 1], fabsf(f.y));
             }
         }
-    }
-    // lanes of equal parity hold the same channels
     #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        #pragma unroll
-        for (int o = 2; o < 32; o <<= 1) m[k] = fmaxf(m[k], __shfl_xor_sync(0xffffffffu, m[k], o));
-    if (lane < 2) {
+    for (int k = 0; k < 8; ++k) {                          // lanes of equal l mod 8 hold the same channels
+        m[k] = fmaxf(m[k], __shfl_xor_sync(0xffffffffu, m[k], 8));
+        m[k] = fmaxf(m[k], __shfl_xor_sync(0xffffffffu, m[k], 16));
+    }
+    if (lane < 8) {
         #pragma unroll
         for (int k = 0; k < 8; ++k) red[warp][8 * lane + k] = m[k];
     }
@@ -252,38 +267,76 @@ __global__ void __launch_bounds__(256) attn_vquant_kernel(AttnArgs a) {
     if (tid < VQ_CH) {
         float mm = 0.f;
         #pragma unroll
-        for (int w = 0; w < 8; ++w) mm = fmaxf(mm, red[w][tid]);
+        for (int w = 0; w < VQ_THREADS / 32; ++w) mm = fmaxf(mm, red[w][tid]);
+        for (int c = 0; c < split; ++c)
+            asm volatile("st.shared::cluster.f32 [%0], %1;"
+                         :: "r"(mapa_shared(smem_addr(&cl_max[rank][tid]), (uint32_t)c)), "f"(mm) : "memory");
+    }
+    cluster_sync();              // nobody touches another CTA's memory after this
+    if (tid < VQ_CH) {
+        float mm = 0.f;
+        for (int c = 0; c < split; ++c) mm = fmaxf(mm, cl_max[c][tid]);
         const bool nz = mm > 0.f;
-        a.t[c0 + tid] = nz ? __fdiv_rn(mm, 7.f) : 0.f;
+        if (rank == 0) a.t[c0 + tid] = nz ? __fdiv_rn(mm, 7.f) : 0.f;
         rcp[tid] = nz ? __fdiv_rn(7.f, mm) : 0.f;
     }
     __syncthreads();
     float rc[8];
     #pragma unroll
-    for (int k = 0; k < 8; ++k) rc[k] = rcp[8 * hv + k];
-    for (int r0 = 0; r0 < a.L; r0 += VQ_KEYS) {
-        uint4 v[4];
+    for (int k = 0; k < 8; ++k) rc[k] = rcp[8 * cg + k];
+    #pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+        if (j >= chunks) break;                            // CTA-uniform
+        if (j > 0) __syncthreads();                        // the previous chunk has left the tile
         #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = load(r0 + rr + 128 * u);
-        #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const T2* p = reinterpret_cast<const T2*>(&v[u]);
+        for (int u = 0; u < 2; ++u) {
+            const int p = pair + 32 * u;
+            const T2* lo = reinterpret_cast<const T2*>(&v[j][2 * u]);
+            const T2* hi = reinterpret_cast<const T2*>(&v[j][2 * u + 1]);
+            const int word = 4 * ((p >> 2) ^ cg) + (p & 3);
             #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float2 f = to_float2(p[k]);
-                tile[8 * hv + 2 * k][rr + 128 * u] = __half_as_ushort(__float2half_rn(rintf(__fmul_rn(f.x, rc[2 * k]))));
-                tile[8 * hv + 2 * k + 1][rr + 128 * u] =
-                    __half_as_ushort(__float2half_rn(rintf(__fmul_rn(f.y, rc[2 * k + 1]))));
+                const float2 f = to_float2(lo[k]), g = to_float2(hi[k]);
+                const __half2 x = __floats2half2_rn(rintf(__fmul_rn(f.x, rc[2 * k])), rintf(__fmul_rn(g.x, rc[2 * k])));
+                const __half2 y = __floats2half2_rn(rintf(__fmul_rn(f.y, rc[2 * k + 1])),
+                                                    rintf(__fmul_rn(g.y, rc[2 * k + 1])));
+                tile[8 * cg + 2 * k][word] = *reinterpret_cast<const uint32_t*>(&x);
+                tile[8 * cg + 2 * k + 1][word] = *reinterpret_cast<const uint32_t*>(&y);
             }
         }
         __syncthreads();
-        const int segs = min(VQ_KEYS, a.L - r0) / 8;          // L is a multiple of 128
-        for (int i = tid; i < VQ_CH * segs; i += 256) {
-            const int c = i / segs, sg = i - c * segs;
-            *reinterpret_cast<uint4*>(a.Vt + (size_t)(c0 + c) * a.L + r0 + 8 * sg) =
-                *reinterpret_cast<const uint4*>(&tile[c][8 * sg]);
+        #pragma unroll
+        for (int i = tid; i < VQ_CH * 16; i += VQ_THREADS) {
+            const int c = i >> 4, g = i & 15;              // keys 8 g .. 8 g + 7 of channel c
+            *reinterpret_cast<uint4*>(a.Vt + (size_t)(c0 + c) * a.L + (chunk0 + j) * ATTN_TILE + 8 * g) =
+                *reinterpret_cast<const uint4*>(&tile[c][4 * (g ^ (c >> 3))]);
         }
-        __syncthreads();
+    }
+}
+
+// A cluster of CTAs per 64 channels: as many as there are chunks of 128 keys,
+// up to 8, each with ceil(chunks / 8) of them.
+template <typename T>
+cudaError_t launch_vquant(const AttnArgs& a, cudaStream_t stream) {
+    const int chunks = a.L / ATTN_TILE, per = (chunks + VQ_MAX_SPLIT - 1) / VQ_MAX_SPLIT;
+    const int nch = per <= 1 ? 1 : per <= 2 ? 2 : per <= 4 ? 4 : 8;     // L <= 8192
+    const int split = (chunks + nch - 1) / nch;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = split;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(ATTN_D * a.Hkv / VQ_CH * split));
+    cfg.blockDim = dim3(VQ_THREADS);
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    switch (nch) {
+        case 1: return cudaLaunchKernelEx(&cfg, attn_vquant_kernel<T, 1>, a, split);
+        case 2: return cudaLaunchKernelEx(&cfg, attn_vquant_kernel<T, 2>, a, split);
+        case 4: return cudaLaunchKernelEx(&cfg, attn_vquant_kernel<T, 4>, a, split);
+        default: return cudaLaunchKernelEx(&cfg, attn_vquant_kernel<T, 8>, a, split);
     }
 }
 
@@ -768,8 +821,7 @@ cudaError_t launch_pv_tac(const AttnArgs& a, cudaStream_t stream) {
         return cudaFuncSetAttribute(attn_pv_tac_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ATT_SMEM);
     });
     if (e != cudaSuccess) return e;
-    attn_vquant_kernel<T><<<Ckv / VQ_CH, 256, 0, stream>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_vquant<T>(a, stream)) != cudaSuccess) return e;
     // persistent CTAs, one per SM at most, each with the same number of
     // items (the last CTAs one fewer)
     const int items = a.L / ATTN_TILE * a.H;
