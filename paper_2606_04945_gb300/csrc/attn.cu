@@ -225,6 +225,8 @@ __global__ void __launch_bounds__(VQ_THREADS) attn_vquant_kernel(AttnArgs a, int
     __shared__ float cl_max[VQ_MAX_SPLIT][VQ_CH];          // the channel maxima of the cluster's CTAs
     __shared__ float rcp[VQ_CH];
     __shared__ __align__(16) uint32_t tile[VQ_CH][ATTN_TILE / 2];
+    grid_dependency_wait();            // launched with programmatic serialisation
+    grid_launch_dependents();
     const int rank = (int)cluster_ctarank();
     const int c0 = ((int)blockIdx.x / split) * VQ_CH;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -322,16 +324,17 @@ cudaError_t launch_vquant(const AttnArgs& a, cudaStream_t stream) {
     const int nch = per <= 1 ? 1 : per <= 2 ? 2 : per <= 4 ? 4 : 8;     // L <= 8192
     const int split = (chunks + nch - 1) / nch;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = split;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1] = pdl_attribute();
     cfg.gridDim = dim3((unsigned)(ATTN_D * a.Hkv / VQ_CH * split));
     cfg.blockDim = dim3(VQ_THREADS);
     cfg.stream = stream;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     switch (nch) {
         case 1: return cudaLaunchKernelEx(&cfg, attn_vquant_kernel<T, 1>, a, split);
         case 2: return cudaLaunchKernelEx(&cfg, attn_vquant_kernel<T, 2>, a, split);
@@ -421,6 +424,10 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
+    // the prologue above overlaps the previous kernel (programmatic launch);
+    // every global access of every role comes after this
+    grid_dependency_wait();
+    grid_launch_dependents();
 
     if (warp == ATT_TMA_WARP) {
         bool ok = true;
@@ -827,8 +834,15 @@ cudaError_t launch_pv_tac(const AttnArgs& a, cudaStream_t stream) {
     const int items = a.L / ATTN_TILE * a.H;
     const int per_cta = (items + num_sms() - 1) / num_sms();
     const int grid = (items + per_cta - 1) / per_cta;
-    attn_pv_tac_kernel<T><<<grid, ATT_THREADS, ATT_SMEM, stream>>>(a, tq, tk, tv, tz);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1] = {pdl_attribute()};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(ATT_THREADS);
+    cfg.dynamicSmemBytes = ATT_SMEM;
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, attn_pv_tac_kernel<T>, a, tq, tk, tv, tz);
 }
 
 cudaError_t launch_attention_pv_tac(const AttnArgs& a, cudaStream_t stream) {
