@@ -430,17 +430,17 @@ template <> struct To<float> { static __device__ __forceinline__ float f(float h
 // every address is a per-thread base plus a constant. Only layout 3 and the
 // row maximum need the whole CTA.
 //
-// Bound by instruction issue (67% of the slots at 8192 x 4096) and shared-
-// memory wavefronts (74%), not by HBM. An earlier split (32 consecutive
+// Bound by instruction issue and shared-memory wavefronts (67% and 74% busy at
+// 8192 x 4096 and seven CTAs per SM), not by HBM. An earlier split (32 consecutive
 // elements per lane first, then two more layouts) staged x and the smoothing
 // vector through shared memory to reach its first layout: 224 wavefronts per
 // 1024 elements instead of 128 (192 with layout 3), and 1141 warp instructions
 // instead of 859 (1349 for the present split with the Hadamard block known
 // only at run time: the branches around the stages keep the register pairs
 // apart). Microseconds back to back, before and now: 8192 x 4096 fp16, hb 4096
-// 43.0, 35.1; 8192 x 3584 bf16, hb 512 39.8, 29.3; 8192 x 18944 245.6, 176.2;
-// 1024 x 12288 23.5, 18.0; 1024 x 4096 8.3, 6.5; codes of 24576 x 4096 weights
-// 120.5, 97.7.
+// 43.0, 33.2; 8192 x 3584 bf16, hb 512 39.8, 29.3; 8192 x 18944 245.6, 166;
+// 1024 x 12288 23.5, 17.6; 1024 x 4096 8.3, 6.5; codes of 24576 x 4096 weights
+// 120.5, 92.0.
 // Butterflies on pairs of registers use the packed f32x2 add and subtract
 // (each half rounds like the scalar operation).
 // ---------------------------------------------------------------------------
@@ -544,8 +544,15 @@ __device__ __forceinline__ void raw4_to_f(const float4& w, float* f) {
 // G2: rows a0.L .. a0.L + b.L - 1 of the grid quantise problem b (the same
 // K, hb, input type and code width; its own X, mask, transform and outputs):
 // two quantisations in one launch.
-template <typename Tin, int HB, bool ASYM, bool CLUSTER, bool G2>
-__global__ void __launch_bounds__(128, 7)
+// FULL (HB 4096): every slice is whole, so no test for missing chunks. Alone it
+// is the shorter code, but its schedule loses in a single wave of CTAs (1024 x
+// 4096: 6.9 us against 6.4), so only launches of several waves take it (8192 x
+// 4096: 33.2 against 35.1; 1024 x 12288 17.6, 18.0).
+// CTAs per SM: seven (72 registers); eight (64, no spills for 16-bit inputs)
+// with FULL, and for clustered rows with blocks of 512 (8192 x 18944: 166 us
+// against 176), but not in a single wave (1000 x 3584: 5.7 against 5.3).
+template <typename Tin, int HB, bool ASYM, bool CLUSTER, bool G2, bool FULL = false>
+__global__ void __launch_bounds__(128, FULL || (HB == 512 && CLUSTER) ? 8 : 7)
 sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
     static_assert(!G2 || !CLUSTER, "grouped launches run one CTA per row");
     using Raw = typename Raw4<Tin>::V;
@@ -569,8 +576,9 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
     const Tin* X = static_cast<const Tin*>(a.X) + (size_t)row * K;
     const int base = rank * 4096;
     const int c0 = base + warp * 1024;                           // first element of the warp's chunk
-    const bool live = c0 < K;
-    const bool half = K - c0 < 1024;      // a last chunk of 512: its upper half is zeros, never stored
+    // a slice may end early, with a last chunk of 512 whose upper half is zeros, never stored
+    const bool live = FULL || c0 < K;
+    const bool half = !FULL && K - c0 < 1024;
     float* own = buf + warp * SLICE + 4 * lane;                  // layout 1: row q at own + QROW q
     float* tr = buf + warp * SLICE + (lane & 3) + QROW * (lane >> 2);   // layout 2: register i at tr + 4 i
 
@@ -637,7 +645,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
         #pragma unroll
         for (int g = 0; g < 8; ++g) {
             ulonglong2 w = make_ulonglong2(0, 0);
-            if (base + (g >> 1) * 1024 < K)                      // chunk g >> 1 exists
+            if (FULL || base + (g >> 1) * 1024 < K)              // chunk g >> 1 exists
                 w = *reinterpret_cast<const ulonglong2*>(buf + (g >> 1) * SLICE + QROW * (2 * warp + (g & 1)) +
                                                          4 * lane);
             p[2 * g] = w.x;
@@ -646,6 +654,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
         reg_stages32(p, 8, hb / 128);                            // h = 1024, 2048
     }
     auto first = [&](int g) { return e_base + (g >> 1) * e_step + (g & 1) * 128; };   // element of group g
+    auto inside = [&](int g) { return FULL || first(g) < K; };
     float v[32];
     #pragma unroll
     for (int i = 0; i < 16; ++i) unpack2f(p[i], v[2 * i], v[2 * i + 1]);
@@ -667,7 +676,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
     if (a.v_dbg != nullptr) {
         #pragma unroll
         for (int g = 0; g < 8; ++g)
-            if (first(g) < K)
+            if (inside(g))
                 *reinterpret_cast<float4*>(a.v_dbg + (size_t)row * K + first(g)) =
                     make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
     }
@@ -743,7 +752,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
             int qi[4];
             codes(g, qf, qi);
             const __half2 h0 = __floats2half2_rn(qf[0], qf[1]), h1 = __floats2half2_rn(qf[2], qf[3]);
-            if (first(g) < K)
+            if (inside(g))
                 *reinterpret_cast<uint2*>(dst + 2 * first(g)) =
                     make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
         }
@@ -754,7 +763,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
             float qf[4];
             int qi[4];
             codes(g, qf, qi);
-            if (first(g) < K) *reinterpret_cast<uint32_t*>(dst + first(g)) = e4m3_bytes4(qf);
+            if (inside(g)) *reinterpret_cast<uint32_t*>(dst + first(g)) = e4m3_bytes4(qf);
         }
     }
     if (a.Xq != nullptr) {
@@ -764,7 +773,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
             float qf[4];
             int qi[4];
             codes(g, qf, qi);
-            if (first(g) >= K) continue;
+            if (!inside(g)) continue;
             if (wide)
                 *reinterpret_cast<uint32_t*>(dst + first(g)) =
                     prmt(prmt((uint32_t)qi[0], (uint32_t)qi[1], 0x0040u),
@@ -796,7 +805,13 @@ cudaError_t launch_rows_kind(const QuantArgs& a, const QuantArgs& b, cudaStream_
     cfg.attrs = at;
     cfg.numAttrs = CLUSTER ? 2 : 1;
     if constexpr (!ASYM) {
-        if (a.hb == 4096) return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2>, a, b, ctas);
+        if (a.hb == 4096) {              // (K is a multiple of 4096)
+            if constexpr (!G2) {
+                if (a.L * ctas > 7 * num_sms())
+                    return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2, true>, a, b, ctas);
+            }
+            return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2>, a, b, ctas);
+        }
         if (a.hb == 512) return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 512, ASYM, CLUSTER, G2>, a, b, ctas);
     }
     return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 0, ASYM, CLUSTER, G2>, a, b, ctas);
