@@ -3,7 +3,8 @@
 //   out[i][b*g + r] = sum_j M[b][r][j] * Z[i][b*g + j] + d[b][r]
 //
 // 16-bit inputs with g = 64 or 128 run on the tensor cores (tac_tc_kernel
-// below). Otherwise, the CUDA-core kernel: grid (token tiles, blocks b). A
+// below), blocks of up to 32 on tac_small_kernel. Otherwise (float32 inputs with
+// g = 64 or 128), the CUDA-core kernel: grid (token tiles, blocks b). A
 // CTA stages M_b transposed (Mt[j][r]) and a tile of TM tokens of block b in shared memory, then each thread computes
 // RT = 4 tokens x RC = 8 channels with float32 FMAs, reading four j at a time
 // (float4) from both tiles. TM = 8192 / g tokens, so the token tile is
@@ -33,7 +34,7 @@ template <> __device__ __forceinline__ float from_f<float>(float x) { return x; 
 template <int G, typename TIn, typename TOut>
 __global__ void __launch_bounds__(TPB)
 tac_kernel(TacArgs a) {
-    constexpr int RC = G < 8 ? G : 8;         // channels per thread
+    constexpr int RC = 8;                     // channels per thread
     constexpr int CG = G / RC;                // channel groups
     constexpr int TG = TPB / CG;              // token groups
     constexpr int RT = 4;                     // tokens per thread
@@ -77,7 +78,7 @@ tac_kernel(TacArgs a) {
             z[t][0] = v.x; z[t][1] = v.y; z[t][2] = v.z; z[t][3] = v.w;
         }
         #pragma unroll
-        for (int jj = 0; jj < 4 && jj < G; ++jj) {
+        for (int jj = 0; jj < 4; ++jj) {
             float m[RC];
             #pragma unroll
             for (int c = 0; c < RC; c += 4) {
@@ -107,8 +108,7 @@ tac_kernel(TacArgs a) {
 
 template <int G, typename TIn, typename TOut>
 cudaError_t launch_g(const TacArgs& a, cudaStream_t stream) {
-    constexpr int RC = G < 8 ? G : 8;
-    constexpr int TM = (TPB / (G / RC)) * 4;
+    constexpr int TM = (TPB / (G / 8)) * 4;
     constexpr size_t smem = (size_t)G * G * 4 + (size_t)TM * (G + 4) * 4;
     static DeviceCache<int> attr;
     int done = 0;
@@ -119,6 +119,160 @@ cudaError_t launch_g(const TacArgs& a, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     dim3 grid((a.L + TM - 1) / TM, a.C / G);
     tac_kernel<G, TIn, TOut><<<grid, TPB, smem, stream>>>(a);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Small blocks, g <= 32: the same float32 sums in the same order as tac_kernel,
+// g FMAs and a quarter as many shared-memory broadcasts per element, which bound
+// it from g = 8 on. A CTA takes 128 channels (128 / g blocks) of a tile of
+// tokens, so that rows are read and written in 256-byte runs (tac_kernel's tile
+// is one block wide: 2-byte loads in rows of 2 g bytes). The tile lies in shared
+// memory as float32, rows padded to 132; a thread takes one block of two tokens
+// (half a tile apart) into registers, so that every M value read serves both,
+// and writes the results back over its inputs. Rows of 132 floats put the
+// 16-byte accesses of eight lanes into different banks.
+// 64 tokens and 128 threads, five CTAs per SM; for g = 32 (one unit per thread
+// needs the wider tile's threads) 128 and 256, two: 77 us against 86.
+// 8192 x 4096 fp16, tac_kernel and now, us: g = 4 349, 42; 8 305, 57; 16 184, 58;
+// 32 165, 77. 1024 x 2560, g = 16: 26.7, 8.3.
+// ---------------------------------------------------------------------------
+constexpr int SM_COLS = 128, SM_ROW = SM_COLS + 4;
+template <int G>
+struct TacSmall {
+    static constexpr int TOKENS = G == 32 ? 128 : 64, THREADS = 2 * TOKENS, CTAS = G == 32 ? 2 : 5;
+    static constexpr size_t SMEM = (size_t)(TOKENS * SM_ROW + SM_COLS * G + SM_COLS) * 4;   // tile, M, d
+};
+
+template <typename T> struct Vec8 {                          // 8 channels of a 16-bit type
+    static __device__ __forceinline__ void load(const T* p, float (&f)[8]) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4*>(p));
+        const T* h = reinterpret_cast<const T*>(&w);
+        #pragma unroll
+        for (int k = 0; k < 8; ++k) f[k] = to_f<T>(h[k]);
+    }
+    static __device__ __forceinline__ void store(T* p, const float (&f)[8]) {
+        uint4 w;
+        T* h = reinterpret_cast<T*>(&w);
+        #pragma unroll
+        for (int k = 0; k < 8; ++k) h[k] = from_f<T>(f[k]);
+        *reinterpret_cast<uint4*>(p) = w;
+    }
+};
+template <> struct Vec8<float> {
+    static __device__ __forceinline__ void load(const float* p, float (&f)[8]) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+        f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+    }
+    static __device__ __forceinline__ void store(float* p, const float (&f)[8]) {
+        reinterpret_cast<float4*>(p)[0] = make_float4(f[0], f[1], f[2], f[3]);
+        reinterpret_cast<float4*>(p)[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+};
+
+template <int G, typename TIn, typename TOut>
+__global__ void __launch_bounds__(TacSmall<G>::THREADS, TacSmall<G>::CTAS)
+tac_small_kernel(TacArgs a) {
+    constexpr int SM_TOKENS = TacSmall<G>::TOKENS, TPB = TacSmall<G>::THREADS;
+    constexpr int BLOCKS = SM_COLS / G;
+    constexpr int PER_ROW = SM_COLS / 8, LOADS = SM_TOKENS * PER_ROW / TPB;      // 8-channel vectors per thread
+    constexpr int UNITS = SM_TOKENS / 2 * BLOCKS / TPB;                          // (block, token pair) per thread
+    static_assert(UNITS >= 1, "at least one unit per thread");
+    extern __shared__ float4 smem4[];
+    float* tile = reinterpret_cast<float*>(smem4);           // [SM_TOKENS][SM_ROW]
+    float* Ms = tile + SM_TOKENS * SM_ROW;                   // [BLOCKS][G][G]
+    float* ds = Ms + SM_COLS * G;                            // [SM_COLS]
+    const int tok0 = blockIdx.x * SM_TOKENS, c0 = blockIdx.y * SM_COLS;
+    const int C = a.C, cols = min(SM_COLS, C - c0);          // a multiple of 8 and of G
+    const TIn* Z = static_cast<const TIn*>(a.Z);
+    TOut* out = static_cast<TOut*>(a.out);
+    const int vc = threadIdx.x % PER_ROW * 8, vr = threadIdx.x / PER_ROW;        // this thread's vectors: rows vr + 16 i
+    float f[LOADS][8];
+    #pragma unroll
+    for (int i = 0; i < LOADS; ++i) {
+        const int tok = tok0 + vr + i * (TPB / PER_ROW);
+        if (tok < a.L && vc < cols) Vec8<TIn>::load(Z + (size_t)tok * C + c0 + vc, f[i]);
+        else {
+            #pragma unroll
+            for (int k = 0; k < 8; ++k) f[i][k] = 0.f;
+        }
+    }
+    for (int i = threadIdx.x; i < cols * G / 4; i += TPB)    // the tile's blocks of M are contiguous
+        reinterpret_cast<float4*>(Ms)[i] = __ldg(reinterpret_cast<const float4*>(a.M + (size_t)c0 * G) + i);
+    for (int i = threadIdx.x; i < cols; i += TPB) ds[i] = a.d ? __ldg(a.d + c0 + i) : 0.f;
+    #pragma unroll
+    for (int i = 0; i < LOADS; ++i) {
+        float4* t = reinterpret_cast<float4*>(tile + (vr + i * (TPB / PER_ROW)) * SM_ROW + vc);
+        t[0] = make_float4(f[i][0], f[i][1], f[i][2], f[i][3]);
+        t[1] = make_float4(f[i][4], f[i][5], f[i][6], f[i][7]);
+    }
+    __syncthreads();
+    #pragma unroll 1
+    for (int u = 0; u < UNITS; ++u) {
+        const int id = threadIdx.x + u * TPB;
+        const int b = id / (SM_TOKENS / 2), t = id % (SM_TOKENS / 2);            // b is warp-uniform
+        if (b * G >= cols) break;
+        float* z0 = tile + t * SM_ROW + b * G;
+        float* z1 = z0 + (SM_TOKENS / 2) * SM_ROW;
+        float x0[G], x1[G];
+        #pragma unroll
+        for (int j = 0; j < G; j += 4) {
+            const float4 p = *reinterpret_cast<const float4*>(z0 + j), q = *reinterpret_cast<const float4*>(z1 + j);
+            x0[j] = p.x; x0[j + 1] = p.y; x0[j + 2] = p.z; x0[j + 3] = p.w;
+            x1[j] = q.x; x1[j + 1] = q.y; x1[j + 2] = q.z; x1[j + 3] = q.w;
+        }
+        const float* m = Ms + b * G * G;
+        #pragma unroll 1
+        for (int r0 = 0; r0 < G; r0 += 4) {
+            float y0[4], y1[4];
+            #pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                y0[r] = y1[r] = 0.f;
+                #pragma unroll
+                for (int j = 0; j < G; j += 4) {
+                    const float4 w = *reinterpret_cast<const float4*>(m + (r0 + r) * G + j);
+                    y0[r] = fmaf(x0[j], w.x, y0[r]);
+                    y0[r] = fmaf(x0[j + 1], w.y, y0[r]);
+                    y0[r] = fmaf(x0[j + 2], w.z, y0[r]);
+                    y0[r] = fmaf(x0[j + 3], w.w, y0[r]);
+                    y1[r] = fmaf(x1[j], w.x, y1[r]);
+                    y1[r] = fmaf(x1[j + 1], w.y, y1[r]);
+                    y1[r] = fmaf(x1[j + 2], w.z, y1[r]);
+                    y1[r] = fmaf(x1[j + 3], w.w, y1[r]);
+                }
+                const float d = ds[b * G + r0 + r];
+                y0[r] += d;
+                y1[r] += d;
+            }
+            *reinterpret_cast<float4*>(z0 + r0) = make_float4(y0[0], y0[1], y0[2], y0[3]);
+            *reinterpret_cast<float4*>(z1 + r0) = make_float4(y1[0], y1[1], y1[2], y1[3]);
+        }
+    }
+    __syncthreads();
+    #pragma unroll
+    for (int i = 0; i < LOADS; ++i) {
+        const int row = vr + i * (TPB / PER_ROW), tok = tok0 + row;
+        if (tok >= a.L || vc >= cols) continue;
+        const float4* t = reinterpret_cast<const float4*>(tile + row * SM_ROW + vc);
+        const float4 p = t[0], q = t[1];
+        const float o[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+        Vec8<TOut>::store(out + (size_t)tok * C + c0 + vc, o);
+    }
+}
+
+template <int G, typename TIn, typename TOut>
+cudaError_t launch_small(const TacArgs& a, cudaStream_t stream) {
+    using P = TacSmall<G>;
+    static DeviceCache<int> attr;
+    int done = 0;
+    const cudaError_t e = attr.get(&done, [](int, int* v) {
+        *v = 1;
+        return cudaFuncSetAttribute(tac_small_kernel<G, TIn, TOut>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)P::SMEM);
+    });
+    if (e != cudaSuccess) return e;
+    dim3 grid((a.L + P::TOKENS - 1) / P::TOKENS, (a.C + SM_COLS - 1) / SM_COLS);
+    tac_small_kernel<G, TIn, TOut><<<grid, P::THREADS, P::SMEM, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -750,10 +904,10 @@ cudaError_t launch_io(const TacArgs& a, cudaStream_t stream) {
         }
     }
     switch (a.g) {
-        case 4: return launch_g<4, TIn, TOut>(a, stream);
-        case 8: return launch_g<8, TIn, TOut>(a, stream);
-        case 16: return launch_g<16, TIn, TOut>(a, stream);
-        case 32: return launch_g<32, TIn, TOut>(a, stream);
+        case 4: return launch_small<4, TIn, TOut>(a, stream);
+        case 8: return launch_small<8, TIn, TOut>(a, stream);
+        case 16: return launch_small<16, TIn, TOut>(a, stream);
+        case 32: return launch_small<32, TIn, TOut>(a, stream);
         case 64: return launch_g<64, TIn, TOut>(a, stream);
         case 128: return launch_g<128, TIn, TOut>(a, stream);
         default: return cudaErrorInvalidValue;
