@@ -280,7 +280,9 @@ int w8_codes_f16(const uint8_t* Wq, int N, int K, uint8_t* We, void* stream);
  *   One 16-bit tensor-core product (tcgen05 kind::f16, CTA pairs) on the
  *   codes, accumulated in float32 in runs of 512 K (each run an integer of
  *   magnitude at most 512 * 127^2 < 2^23, so exact); the epilogue adds the
- *   runs in int32.
+ *   runs in int32. With few tokens (up to 256, where it is faster) K is split
+ *   over up to eight CTAs per 128 channels instead, in runs of at most 1024 K
+ *   (below 2^24), likewise added in int32: the same results.
  *   s_a [L], s_w [N] float32; bias [N] float32 or NULL.
  *   Y  [L][N] out, y_dtype F16, BF16 or F32, 16-byte aligned.
  *   acc_dbg [L][N] int32 out (the exact accumulators) or NULL.
@@ -473,8 +475,9 @@ int starq_last_gemm_tile(void);
  * fp16_gemm_ref -- the 16-bit baseline of the projections: C = A B^T with
  * float32 accumulation and one rounding to the element type. It is the
  * unquantised model's linear layer that Sec. 4.4 measures its speed-up
- * against; here it serves only as that denominator (the same CTA-pair
- * tcgen05 kernel structure as w4a4_gemm, kind::f16, no cuBLAS).
+ * against; here it serves only as that denominator (the same tcgen05 kernels
+ * as w4a4_gemm, CTA pairs or the few-token one that splits K, kind::f16, no
+ * cuBLAS; the order of the float32 sums is the kernel's).
  *
  *   A [M][K], B [N][K] row-major, C [M][N] out; all of element type dtype
  *   (F16 or BF16), 16-byte aligned.

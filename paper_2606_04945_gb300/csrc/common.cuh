@@ -73,10 +73,11 @@ struct GemmArgs {
     int swiglu = 0;
 };
 cudaError_t launch_w4a4_gemm(const GemmArgs& a, cudaStream_t stream);
-// The same product with Xe and We for few tokens (few_tokens(a)): K split over
-// a cluster of *split CTAs per 128-channel tile.
-bool few_tokens(const GemmArgs& a);
-cudaError_t launch_w4a4_gemm_few(const GemmArgs& a, int* split, cudaStream_t stream);
+// The same product with Xe and We for few tokens (few_tokens(a, opk)): K split
+// over a cluster of *split CTAs per 128-channel tile. opk: 0 E4M3 codes, 1 fp16,
+// 2 bf16 (plain products), 3 8-bit codes held as fp16.
+bool few_tokens(const GemmArgs& a, int opk);
+cudaError_t launch_gemm_few(const GemmArgs& a, int opk, int* split, cudaStream_t stream);
 // Two independent products in one persistent TMA pair launch (the same L,
 // K and output type; Xe and We given for both; no SwiGLU).
 cudaError_t launch_w4a4_gemm_grouped(const GemmArgs& a, const GemmArgs& b, cudaStream_t stream);

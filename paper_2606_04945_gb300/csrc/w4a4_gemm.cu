@@ -1596,8 +1596,20 @@ cudaError_t launch_unpack_e4m3(const uint8_t* packed, uint8_t* e4m3, size_t rows
 
 int last_gemm_tile() { return g_last_tile; }
 
+// The few-token kernel where it is the faster one (a cap on the CTA pairs asks
+// for the pair kernel).
+static bool takes_few(const GemmArgs& a, int opk) { return g_pair_limit == 0 && few_tokens(a, opk); }
+static cudaError_t launch_few_tile(const GemmArgs& a, int opk, cudaStream_t stream) {
+    int split = 0;
+    const cudaError_t e = launch_gemm_few(a, opk, &split, stream);
+    if (e == cudaSuccess) g_last_tile = 128 * 10 + split;
+    return e;
+}
+
 cudaError_t launch_fp16_gemm(const GemmArgs& a, cudaStream_t stream) {
     if (a.L == 0) return cudaSuccess;
+    const int opk = a.y_dtype == STARQ_BF16 ? 2 : 1;
+    if (takes_few(a, opk)) return launch_few_tile(a, opk, stream);
     switch (a.y_dtype) {
         case STARQ_F16: return launch_tma_typed<__half, 1>(a, stream);
         case STARQ_BF16: return launch_tma_typed<__nv_bfloat16, 2>(a, stream);
@@ -1608,6 +1620,7 @@ cudaError_t launch_fp16_gemm(const GemmArgs& a, cudaStream_t stream) {
 cudaError_t launch_w8a8_gemm(const GemmArgs& a, cudaStream_t stream) {
     if (a.L == 0) return cudaSuccess;
     if (a.Xe == nullptr || a.We == nullptr || a.swiglu) return cudaErrorInvalidValue;
+    if (takes_few(a, 3)) return launch_few_tile(a, 3, stream);
     switch (a.y_dtype) {
         case STARQ_F16: return launch_tma_typed<__half, 3>(a, stream);
         case STARQ_BF16: return launch_tma_typed<__nv_bfloat16, 3>(a, stream);
@@ -1638,12 +1651,7 @@ cudaError_t launch_w4a4_gemm_grouped(const GemmArgs& a, const GemmArgs& b, cudaS
 cudaError_t launch_w4a4_gemm(const GemmArgs& a, cudaStream_t stream) {
     if (a.L == 0) return cudaSuccess;
     if (a.Xe != nullptr && a.We != nullptr) {
-        if (g_pair_limit == 0 && few_tokens(a)) {      // (a cap on the CTA pairs asks for the pair kernel)
-            int split = 0;
-            const cudaError_t e = launch_w4a4_gemm_few(a, &split, stream);
-            if (e == cudaSuccess) g_last_tile = 128 * 10 + split;
-            return e;
-        }
+        if (takes_few(a, 0)) return launch_few_tile(a, 0, stream);
         switch (a.y_dtype) {
             case STARQ_F16: return launch_tma_typed<__half>(a, stream);
             case STARQ_BF16: return launch_tma_typed<__nv_bfloat16>(a, stream);

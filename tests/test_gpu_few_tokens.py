@@ -85,3 +85,61 @@ def test_few_tokens_swiglu(abi, L, K, F, dtype):
         assert (abi.last_gemm_tile()[0] == 128) == (limit == 0)
         out.append(Hb)
     assert torch.equal(out[0], out[1])
+
+
+# 8-bit codes held as fp16: one accumulator per part (16 stages of 64 K), two, a part that ends
+# inside its second one, the largest magnitudes, and one part per tile
+@pytest.mark.parametrize("L,N,K,out,extreme", [(1, 128, 128, "f16", False), (32, 512, 4096, "bf16", False),
+                                               (17, 1024, 12288, "f16", True), (70, 256, 8320, "f32", False),
+                                               (128, 4096, 4096, "f16", False), (9, 40960, 1024, "f16", True)])
+def test_few_tokens_8bit_exact(abi, L, N, K, out, extreme):
+    rng = np.random.default_rng(L + N + K)
+    draw = (lambda r: np.full((r, K), 127) * rng.choice([-1, 1], (r, 1))) if extreme else \
+        (lambda r: rng.integers(-127, 128, (r, K)))
+    qa, qw = draw(L).astype(np.int64), draw(N).astype(np.int64)
+    s_a, s_w = rng.uniform(0.01, 1, L).astype(np.float32), rng.uniform(0.01, 1, N).astype(np.float32)
+    bias = rng.normal(0, 0.1, N).astype(np.float32) if L == 32 else None
+    Xe, We = H.dev(qa.astype(np.float16)), H.dev(qw.astype(np.float16))
+    res = []
+    for limit in (0, 10 ** 6):
+        prev = abi.set_gemm_pair_limit(limit)
+        try:
+            Y = torch.empty(L, N, dtype=H.torch_dtype(out), device="cuda")
+            acc = torch.empty(L, N, dtype=torch.int32, device="cuda")
+            abi.w8a8_gemm(Xe, H.dev(s_a), We, H.dev(s_w), Y, bias=None if bias is None else H.dev(bias), acc_dbg=acc)
+            abi.check_status()
+        finally:
+            abi.set_gemm_pair_limit(prev)
+        assert (abi.last_gemm_tile()[0] == 128) == (limit == 0)
+        res.append((Y, acc))
+    ref = (qa.astype(np.float64) @ qw.T.astype(np.float64)).astype(np.int64)       # exact below 2^53
+    assert np.array_equal(res[0][1].cpu().numpy(), ref)
+    assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
+
+
+@pytest.mark.parametrize("L,N,K,dt", [(1, 32, 64, "f16"), (20, 4096, 4096, "f16"), (33, 160, 2112, "bf16"),
+                                      (100, 1024, 8192, "bf16"), (64, 512, 16384, "f16")])
+def test_few_tokens_16bit(abi, L, N, K, dt):
+    """Plain 16-bit product: float32 sums of K / split terms and their sum over
+    at most eight parts stay within the bound of one chain of K, and the error
+    against float64 is no larger than the pair kernel's (5 % for the draw)."""
+    rng = np.random.default_rng(L + N + K)
+    rnd = (lambda x: x.astype(np.float16).astype(np.float32)) if dt == "f16" else inputs.round_to_bf16
+    A, B = (rnd(rng.standard_normal((r, K)).astype(np.float32)) for r in (L, N))
+    ref = A.astype(np.float64) @ B.astype(np.float64).T
+    mag = np.abs(A).astype(np.float64) @ np.abs(B).astype(np.float64).T
+    err = []
+    for limit in (0, 10 ** 6):
+        prev = abi.set_gemm_pair_limit(limit)
+        try:
+            C = torch.empty(L, N, dtype=H.torch_dtype(dt), device="cuda")
+            abi.fp16_gemm_ref(H.dev(A, H.torch_dtype(dt)), H.dev(B, H.torch_dtype(dt)), C)
+            abi.check_status()
+        finally:
+            abi.set_gemm_pair_limit(prev)
+        assert (abi.last_gemm_tile()[0] == 128) == (limit == 0)
+        got = H.host(C).astype(np.float64)
+        tol = np.maximum(H.half_spacing(ref, dt), 2.0 ** -11 * np.abs(ref) if dt == "f16" else 0) + 2.0 ** -22 * np.sqrt(K) * mag
+        assert np.all(np.abs(got - ref) <= tol)
+        err.append(np.linalg.norm(got - ref))
+    assert err[0] <= 1.05 * err[1]
