@@ -38,7 +38,7 @@
 //                      with the A operand (Q, P, Z_hat) in tensor memory and
 //                      B (K, V, M) in shared memory.
 //   prologue  the softmax warps copy the Q tile (loaded by TMA) into TMEM.
-//   pass 1  S = Q K^T chunk by chunk (128 keys, two TMEM buffers); each
+//   pass 1  S = Q K^T chunk by chunk (128 keys, three TMEM buffers); each
 //           thread keeps the running maximum of its row's part of S.
 //   pass 2  S again; each thread turns its 32 scores into
 //           e = exp2(s c - m c), c = log2(e) / sqrt(d) (one fma, ex2.approx),
@@ -57,8 +57,9 @@
 // six 32 KB tiles streams each item's Q tile, pass-1 K chunks, pass-2 K and
 // V chunks, M's two halves and then the slot of its output boxes, in the
 // order they are used, running on into the next item.
-// TMEM (512 columns): two S / P buffers, the P V^T accumulator (then the
-// TAC accumulator), Q, and Z_hat's halves (see the column map below). The
+// TMEM (512 columns): two S / P buffers, the P V^T accumulator (a third S
+// buffer in pass 1, then the TAC accumulator), Q, and Z_hat's halves (see the
+// column map below). The
 // tensor pipe keeps almost no queue of issued MMAs, so it runs dry
 // whenever the issuing thread is busy elsewhere (its waits and bookkeeping,
 // slowed by the softmax warps that share its scheduler): the MMA warp
@@ -68,6 +69,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <cstddef>
 #include <type_traits>
 
 #include "attn.cuh"
@@ -96,12 +98,19 @@ constexpr int ATT_TILES_BYTES = ATT_SLOTS * TILE_BYTES;
 // half of the second S buffer. The first S buffer and the lower half of the
 // second stay free, so the next item's Q K^T can follow the TAC product at
 // once (the MMAs of one thread run in issue order, so it cannot overwrite
-// Z_lo before the TAC product has read it).
+// Z_lo before the TAC product has read it). In pass 1 nothing is accumulated
+// yet, so the accumulator's columns are a third S buffer: the softmax warps
+// release it (s_empty[2]) when they have read the previous item's TAC
+// accumulator, and P V^T of chunk 0 follows only their arrivals for P(0),
+// which come after they have read all of pass 1. Three buffers and the
+// bookkeeping below, against two and divided entry numbers (us): 1024 keys x
+// 32 heads 32.8 -> 32.5; 2048 x 28 70.0 -> 68.4; 4096 x 32 297 -> 290; the
+// three buffers with their number taken as it mod 3: 33.4, 71.3, 304.
 constexpr uint32_t TM_S = 0, TM_O = 256, TM_Q = 384;
 constexpr uint32_t TM_TAC = TM_O, TM_ZHI = 448, TM_ZLO = 192;
 
 struct AttSm {
-    uint64_t q_full, full[ATT_SLOTS], empty[ATT_SLOTS], s_full[2], s_empty[2];
+    uint64_t q_full, full[ATT_SLOTS], empty[ATT_SLOTS], s_full[3], s_empty[3];
     uint64_t pv_done, z_full, tac_done;
     uint32_t tmem_base;
     int abort;
@@ -389,16 +398,14 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
     auto use_parity = [](int g) { return ((uint32_t)g / ATT_SLOTS) & 1u; };
     auto item_q0 = [=](int i) { return ((int)blockIdx.x + i * (int)gridDim.x) % nk * ATTN_TILE; };
     auto item_h = [=](int i) { return ((int)blockIdx.x + i * (int)gridDim.x) / nk; };
-    // S buffer of Q K^T number it of item i (pass 1: it = 0 .. nk-1; pass
-    // 2: it = nk + j; the two buffers alternate within each pass) and the
-    // number of that buffer's earlier uses, counted over all items
-    const int u0 = (nk + 1) / 2, u1 = nk / 2;                // uses of buffer 0 / 1 per pass
-    auto sbuf = [=](int i, int it, int& b, int& n) {
-        const int j = it < nk ? it : it - nk;
-        b = j & 1;
-        const int per = b == 0 ? u0 : u1;
-        n = (j >> 1) + (it < nk ? 0 : per) + i * 2 * per;
-    };
+    // The per-chunk bookkeeping of the waiting warps sits on the critical path
+    // (about 80 cycles a chunk for 20 instructions), so it is kept to a few
+    // bits: pass 1 goes round the three S buffers, pass 2 alternates between the
+    // first two (chunk j: buffer j & 1), a mask holds the parity of each buffer's
+    // uses so far, and the MMA warp walks the ring with cursors instead of
+    // dividing entry numbers.
+    auto s_full_bar = [=](int b) { return B(sh->s_full[0]) + 8u * (uint32_t)b; };
+    auto s_empty_bar = [=](int b) { return B(sh->s_empty[0]) + 8u * (uint32_t)b; };
 
     if (threadIdx.x == 0) {
         mbar_init(B(sh->q_full), ATT_SOFTMAX_WARPS);
@@ -406,7 +413,7 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
             mbar_init(B(sh->full[k]), 1);
             mbar_init(B(sh->empty[k]), 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < 3; ++b) {
             mbar_init(B(sh->s_full[b]), 1);
             mbar_init(B(sh->s_empty[b]), ATT_SOFTMAX_WARPS);
         }
@@ -496,6 +503,22 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
                 mma_f16_ts(d, ta + ac, bd + (uint64_t)(koff >> 4), idesc, (acc0 || ks > 0) ? 1u : 0u);
             }
         };
+        // a ring entry: its full barrier (the empty one EMPTY_OFF after it), the
+        // parity of that use, its tile
+        struct Cursor { uint32_t full, parity, tile; };
+        constexpr uint32_t EMPTY_OFF = offsetof(AttSm, empty) - offsetof(AttSm, full);
+        const uint32_t full_end = B(sh->full[0]) + 8u * ATT_SLOTS;
+        auto cursor = [=](int g) { return Cursor{full_bar(g), use_parity(g), slot(g)}; };
+        auto advance = [=](Cursor& c, uint32_t by) {                 // by <= ATT_SLOTS entries
+            c.full += 8u * by;
+            c.tile += (uint32_t)TILE_BYTES * by;
+            if (c.full >= full_end) {
+                c.full -= 8u * ATT_SLOTS;
+                c.tile -= (uint32_t)ATT_TILES_BYTES;
+                c.parity ^= 1u;
+            }
+        };
+        uint32_t uses = 0;
         bool ok = true;
         int tac_commits = 0;
         tc_fence_after();
@@ -505,20 +528,16 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
             ok = mbar_wait_bounded_warp(B(sh->q_full), (uint32_t)(i & 1), abort);
             if (ok && elect_one()) mbar_arrive(empty_bar(gq));
             __syncwarp();
-            // Q K^T number it, once its K tile has landed and the softmax
-            // warps have read the S buffer's previous scores (s_empty)
-            auto qk = [=](int it) -> bool {
-                const int g = g0 + (it < nk ? it : nk + 2 * (it - nk));
-                int b, n;
-                sbuf(i, it, b, n);
-                if (!mbar_wait2_bounded_warp(full_bar(g), use_parity(g), B(sh->s_empty[b]), (uint32_t)(n & 1) ^ 1u,
-                                             abort))
-                    return false;
+            // Q K^T into S buffer b (uses: the parities of the buffers' uses),
+            // once its K tile at c has landed and the softmax warps have read
+            // the buffer's previous scores (s_empty)
+            auto qk = [=](Cursor c, int b, uint32_t uses) -> bool {
+                if (!mbar_wait2_bounded_warp(c.full, c.parity, s_empty_bar(b), (uses >> b & 1u) ^ 1u, abort)) return false;
                 tc_fence_after();
                 if (elect_one()) {
-                    mma_tile(tmem + TM_S + b * ATTN_TILE, TM_Q, slot(g), false, false, IDESC_T);
-                    tc_commit(empty_bar(g));
-                    tc_commit(B(sh->s_full[b]));
+                    mma_tile(tmem + TM_S + b * ATTN_TILE, TM_Q, c.tile, false, false, IDESC_T);
+                    tc_commit(c.full + EMPTY_OFF);
+                    tc_commit(s_full_bar(b));
                 }
                 __syncwarp();
                 return true;
@@ -530,32 +549,47 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
             // landed. Every wait of the issuing thread lets the tensor pipe
             // run dry, so the two products go out back to back behind a
             // single wait.
-            auto step2 = [=](int j) -> bool {
-                const int gv = g0 + nk + 2 * j + 1, gk = gv + 3;
-                const bool more = j + 2 < nk;
-                int b, n;
-                sbuf(i, nk + j, b, n);
-                if (!(more ? mbar_wait3_bounded_warp(B(sh->s_empty[b]), (uint32_t)(n & 1), full_bar(gv), use_parity(gv),
-                                                     full_bar(gk), use_parity(gk), abort)
-                           : mbar_wait2_bounded_warp(B(sh->s_empty[b]), (uint32_t)(n & 1), full_bar(gv), use_parity(gv),
-                                                     abort)))
+            auto step2 = [=](Cursor cv, Cursor ck, int b, uint32_t uses, bool first, bool more) -> bool {
+                const uint32_t sp = (uses >> b & 1u) ^ 1u;
+                if (!(more ? mbar_wait3_bounded_warp(s_empty_bar(b), sp, cv.full, cv.parity, ck.full, ck.parity, abort)
+                           : mbar_wait2_bounded_warp(s_empty_bar(b), sp, cv.full, cv.parity, abort)))
                     return false;
                 tc_fence_after();
                 if (elect_one()) {
-                    mma_tile(tmem + TM_O, TM_S + b * ATTN_TILE, slot(gv), j > 0, true, IDESC_F16);
-                    tc_commit(empty_bar(gv));
+                    mma_tile(tmem + TM_O, TM_S + b * ATTN_TILE, cv.tile, !first, true, IDESC_F16);
+                    tc_commit(cv.full + EMPTY_OFF);
                     if (more) {
-                        mma_tile(tmem + TM_S + b * ATTN_TILE, TM_Q, slot(gk), false, false, IDESC_T);
-                        tc_commit(empty_bar(gk));
-                        tc_commit(B(sh->s_full[b]));
+                        mma_tile(tmem + TM_S + b * ATTN_TILE, TM_Q, ck.tile, false, false, IDESC_T);
+                        tc_commit(ck.full + EMPTY_OFF);
+                        tc_commit(s_full_bar(b));
                     }
                 }
                 __syncwarp();
                 return true;
             };
             tc_fence_after();
-            for (int it = 0; it < nk + 2 && it < 2 * nk && ok; ++it) ok = qk(it);   // pass 1, then two chunks ahead
-            for (int j = 0; j < nk && ok; ++j) ok = step2(j);
+            Cursor c = cursor(g0);
+            for (int it = 0, b = 0; it < nk && ok; ++it) {           // pass 1
+                ok = qk(c, b, uses);
+                uses ^= 1u << b;
+                b = b == 2 ? 0 : b + 1;
+                advance(c, 1);
+            }
+            uses ^= 4u;                                              // (the TAC accumulator's release)
+            Cursor cv = c, ck = c;                                   // pass 2, first two chunks ahead
+            for (int j = 0; j < 2 && j < nk && ok; ++j) {
+                ok = qk(ck, j, uses);
+                uses ^= 1u << j;
+                advance(ck, 2);
+            }
+            advance(cv, 1);
+            for (int j = 0; j < nk && ok; ++j) {
+                const bool more = j + 2 < nk;
+                ok = step2(cv, ck, j & 1, uses, j == 0, more);
+                if (more) uses ^= 1u << (j & 1);
+                advance(cv, 2);
+                advance(ck, 2);
+            }
             if (elect_one()) tc_commit(B(sh->pv_done));
             __syncwarp();
             const int gm = g0 + 3 * nk;               // M_hi; M_lo at gm + 1
@@ -611,6 +645,7 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
             if (lane == 0) mbar_arrive(B(sh->q_full));
             return true;
         };
+        uint32_t uses = 0;                                  // parities of the S buffers' uses
         if (my_items > 0) ok = put_q(0);
         // Every softmax warp runs every item and every named barrier; after a
         // failed wait it only skips the work.
@@ -624,16 +659,16 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
             }
             // pass 1: row maxima
             float mx = -INFINITY;
-            for (int it = 0; it < nk && ok; ++it) {
-                int b, n;
-                sbuf(i, it, b, n);
-                if (!mbar_wait_bounded_warp(B(sh->s_full[b]), (uint32_t)(n & 1), abort)) { ok = false; break; }
+            for (int it = 0, b = 0; it < nk && ok; ++it) {
+                if (!mbar_wait_bounded_warp(s_full_bar(b), uses >> b & 1u, abort)) { ok = false; break; }
+                uses ^= 1u << b;
                 tc_fence_after();
                 tmem_ld_32x32b_x32(tl + TM_S + b * ATTN_TILE + col, r);
                 tmem_ld_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(B(sh->s_empty[b]));
+                if (lane == 0) mbar_arrive(s_empty_bar(b));
+                b = b == 2 ? 0 : b + 1;
                 #pragma unroll
                 for (int k = 0; k < 32; ++k) mx = fmaxf(mx, __uint_as_float(r[k]));
             }
@@ -651,9 +686,9 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
             // decisions move only within 3e-4 of a half-integer)
             const float mxc = __fmul_rn(mx, EXP_SCALE);
             for (int j = 0; j < nk && ok; ++j) {
-                int b, n;
-                sbuf(i, nk + j, b, n);
-                if (!mbar_wait_bounded_warp(B(sh->s_full[b]), (uint32_t)(n & 1), abort)) { ok = false; break; }
+                const int b = j & 1;
+                if (!mbar_wait_bounded_warp(s_full_bar(b), uses >> b & 1u, abort)) { ok = false; break; }
+                uses ^= 1u << b;
                 tc_fence_after();
                 tmem_ld_32x32b_x32(tl + TM_S + b * ATTN_TILE + col, r);
                 tmem_ld_wait();
@@ -689,7 +724,7 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(B(sh->s_empty[b]));
+                if (lane == 0) mbar_arrive(s_empty_bar(b));
             }
             sh->xm[part][row] = (lpa.x + lpb.x) + (lpa.y + lpb.y);
             named_sync_softmax();
@@ -752,6 +787,9 @@ attn_pv_tac_kernel(AttnArgs a, const __grid_constant__ CUtensorMap tm_q, const _
                 tc_fence_after();
                 tmem_ld_32x32b_x32(tl + TM_TAC + col, r);
                 tmem_ld_wait();
+                tc_fence_before();                           // the next item's third S buffer
+                __syncwarp();
+                if (lane == 0) mbar_arrive(s_empty_bar(2));
                 const uint32_t box = slot(go) + (uint32_t)warp * 2048;
                 const bool add_d = a.d != nullptr;
                 #pragma unroll
