@@ -422,7 +422,10 @@ template <> struct To<float> { static __device__ __forceinline__ float f(float h
 //             stages h = 4 .. 64;
 //   layout 3  hb > 1024 only: bits 0, 1, 7 and the chunk number (register
 //             8 j + 4 q + k: element 256 w + 128 q + 4 l + k of chunk j for
-//             lane l of warp w): stages h = 1024, 2048.
+//             lane l of warp w): stages h = 1024, 2048. With blocks of 2048 a
+//             pair of chunks is exchanged between its own two warps (bits 0,
+//             1, 7, 8 and the chunk's), so that of rows of 2048 the other two
+//             stay idle.
 //
 // The layouts change through the warp's own slice of shared memory, eight
 // rows (q) of 128 floats padded to 132: the 16-byte accesses of layouts 1 and
@@ -440,7 +443,10 @@ template <> struct To<float> { static __device__ __forceinline__ float f(float h
 // apart). Microseconds back to back, before and now: 8192 x 4096 fp16, hb 4096
 // 43.0, 33.2; 8192 x 3584 bf16, hb 512 39.8, 29.3; 8192 x 18944 245.6, 166;
 // 1024 x 12288 23.5, 17.6; 1024 x 4096 8.3, 6.5; codes of 24576 x 4096 weights
-// 120.5, 92.0.
+// 120.5, 92.0; asymmetric 8192 x 4096 47.3, 39.7. Rows shorter than a slice
+// (warps without a chunk leave before the codes), with the idle warps working and
+// now: 8192 x 1024 24.7, 18.6; 8192 x 2048 33.2, 24.4; asymmetric 31.8, 20.9 and
+// 39.5, 27.5.
 // Butterflies on pairs of registers use the packed f32x2 add and subtract
 // (each half rounds like the scalar operation).
 // ---------------------------------------------------------------------------
@@ -637,7 +643,21 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
     }
     // group g of four registers: elements e_base + (g >> 1) e_step + 128 (g & 1) ..
     int e_base = c0 + 4 * lane, e_step = 256;
-    if (hb > 1024) {                                             // layout 1 -> 3
+    if (HB == 2048) {                                            // layout 1 -> 3, two chunks (K is a multiple of 2048)
+        e_base = base + 2048 * (warp >> 1) + 512 * (warp & 1) + 4 * lane;
+        if (live) put_own();
+        __syncthreads();
+        if (live) {
+            #pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(
+                    buf + (2 * (warp >> 1) + (g >> 2)) * SLICE + QROW * (4 * (warp & 1) + (g & 3)) + 4 * lane);
+                p[2 * g] = w.x;
+                p[2 * g + 1] = w.y;
+            }
+            reg_stages32(p, 16, 32);                             // h = 1024
+        }
+    } else if (hb > 1024) {                                      // layout 1 -> 3
         e_base = base + warp * 256 + 4 * lane;
         e_step = 1024;
         if (live) put_own();
@@ -653,12 +673,17 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
         }
         reg_stages32(p, 8, hb / 128);                            // h = 1024, 2048
     }
-    auto first = [&](int g) { return e_base + (g >> 1) * e_step + (g & 1) * 128; };   // element of group g
+    auto first = [&](int g) {                                    // element of group g
+        return HB == 2048 ? e_base + (g >> 2) * 1024 + (g & 3) * 128 : e_base + (g >> 1) * e_step + (g & 1) * 128;
+    };
     auto inside = [&](int g) { return FULL || first(g) < K; };
+    // a warp without a chunk has nothing to quantise unless layout 3 gives it a
+    // part of the others' (of rows of 1024 three warps in four are idle)
+    const bool idle = HB != 4096 && !live && (hb <= 1024 || HB == 2048);
     float v[32];
     #pragma unroll
     for (int i = 0; i < 16; ++i) unpack2f(p[i], v[2 * i], v[2 * i + 1]);
-    if (first(7) + 4 > a.d_sh) {          // the lane reaches past the shared coordinates: the gate
+    if (!idle && first(7) + 4 > a.d_sh) {          // the lane reaches past the shared coordinates: the gate
         const int own_lo = masked ? a.d_sh : a.d_sh + a.d_m;
         const int own_hi = masked ? a.d_sh + a.d_m : K;
         #pragma unroll
@@ -743,7 +768,24 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
             }
         }
     };
-    const bool wide = !ASYM && a.qmax > 15;                      // 8-bit codes: fp16 and bytes
+    if (idle) return;                                            // (no barrier follows)
+    if (ASYM) {                                                  // E4M3 bytes and unsigned nibbles, the codes once
+        uint8_t* e4 = a.Xe == nullptr ? nullptr : a.Xe + (size_t)row * (K + 128);
+        uint8_t* nib = a.Xq == nullptr ? nullptr : a.Xq + (size_t)row * (K / 2);
+        #pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            if (HB != 4096 && HB != 2048 && !inside(g)) continue;    // (warp-uniform)
+            float qf[4];
+            int qi[4];
+            codes(g, qf, qi);
+            if (e4 != nullptr) *reinterpret_cast<uint32_t*>(e4 + first(g)) = e4m3_bytes4(qf);
+            if (nib != nullptr)
+                *reinterpret_cast<uint16_t*>(nib + first(g) / 2) =
+                    (uint16_t)(qi[0] | qi[1] << 4 | qi[2] << 8 | qi[3] << 12);
+        }
+        return;
+    }
+    const bool wide = a.qmax > 15;                               // 8-bit codes: fp16 and bytes
     if (a.Xe != nullptr && wide) {
         uint8_t* dst = a.Xe + (size_t)row * K * 2;
         #pragma unroll
@@ -757,7 +799,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
                     make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
         }
     } else if (a.Xe != nullptr) {                                // E4M3 bytes
-        uint8_t* dst = a.Xe + (size_t)row * (ASYM ? K + 128 : K);
+        uint8_t* dst = a.Xe + (size_t)row * K;
         #pragma unroll
         for (int g = 0; g < 8; ++g) {
             float qf[4];
@@ -778,7 +820,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
                 *reinterpret_cast<uint32_t*>(dst + first(g)) =
                     prmt(prmt((uint32_t)qi[0], (uint32_t)qi[1], 0x0040u),
                          prmt((uint32_t)qi[2], (uint32_t)qi[3], 0x0040u), 0x5410u);
-            else                         // (unsigned codes up to 15 when ASYM)
+            else
                 *reinterpret_cast<uint16_t*>(dst + first(g) / 2) =
                     (uint16_t)((qi[0] & 15) | (qi[1] & 15) << 4 | (qi[2] & 15) << 8 | (qi[3] & 15) << 12);
         }
@@ -787,8 +829,9 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
 
 // One launch of the row kernel: a CTA per row (b != nullptr: the rows of b
 // after those of a), or beyond 4096 features a cluster of CTAs per row, one
-// 4096-feature slice each. The blocks of the model widths (512 of 3584 and
-// 18944, 4096 of 4096 and 12288) are compiled in.
+// 4096-feature slice each. Blocks of 512 to 4096 are compiled in (8192 x 4096,
+// hb 1024: 30.2 us, against 33.9 with the block at run time; asymmetric, hb 4096,
+// 45.4 and 52.4).
 template <typename Tin, bool ASYM, bool CLUSTER, bool G2>
 cudaError_t launch_rows_kind(const QuantArgs& a, const QuantArgs& b, cudaStream_t stream) {
     const int ctas = (a.K + 4095) / 4096;
@@ -804,15 +847,20 @@ cudaError_t launch_rows_kind(const QuantArgs& a, const QuantArgs& b, cudaStream_
     cfg.stream = stream;
     cfg.attrs = at;
     cfg.numAttrs = CLUSTER ? 2 : 1;
-    if constexpr (!ASYM) {
-        if (a.hb == 4096) {              // (K is a multiple of 4096)
-            if constexpr (!G2) {
-                if (a.L * ctas > 7 * num_sms())
-                    return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2, true>, a, b, ctas);
-            }
-            return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2>, a, b, ctas);
+    if (a.hb == 4096) {                  // (K is a multiple of 4096)
+        if constexpr (!G2) {
+            if (a.L * ctas > 7 * num_sms())
+                return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2, true>, a, b, ctas);
         }
-        if (a.hb == 512) return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 512, ASYM, CLUSTER, G2>, a, b, ctas);
+        return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 4096, ASYM, CLUSTER, G2>, a, b, ctas);
+    }
+    if (a.hb == 512) return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 512, ASYM, CLUSTER, G2>, a, b, ctas);
+    if constexpr (!G2) {
+        switch (a.hb) {
+            case 1024: return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 1024, ASYM, CLUSTER, G2>, a, b, ctas);
+            case 2048: return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 2048, ASYM, CLUSTER, G2>, a, b, ctas);
+            default: break;
+        }
     }
     return cudaLaunchKernelEx(&cfg, sgat_quant_rows_kernel<Tin, 0, ASYM, CLUSTER, G2>, a, b, ctas);
 }

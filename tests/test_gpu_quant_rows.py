@@ -51,3 +51,28 @@ def test_rows_bitexact(abi, K, hb, dtype, bits):
         assert np.array_equal(Xq.cpu().numpy().view(np.int8), codes)
         value = Xe.view(torch.float16).float().cpu().numpy()
     assert np.array_equal(value, codes.astype(np.float32))
+
+
+# the compiled-in blocks in the asymmetric mode: one wave and several (whole
+# slices only), rows of one CTA and of clusters, half chunks
+@pytest.mark.parametrize("L,K,hb,dtype", [(3, 4096, 4096, "f32"), (1100, 4096, 4096, "f16"), (1300, 4096, 4096, "bf16"),
+                                          (6, 3584, 512, "bf16"), (5, 7680, 512, "f16"), (7, 4608, 512, "f32"),
+                                          (6, 1024, 1024, "f16"), (5, 7168, 1024, "bf16"), (6, 2048, 2048, "f16"),
+                                          (5, 6144, 2048, "bf16"), (4, 1536, 256, "f16")])
+def test_rows_asym_bitexact(abi, L, K, hb, dtype):
+    case = inputs.random_linear(K + L, L, K, 32, dtype="f16" if dtype == "f32" else dtype, hb=hb)
+    xf = case.xf
+    X = H.dev(case.X, H.torch_dtype(dtype))
+    Xq = torch.empty(L, K // 2, dtype=torch.uint8, device="cuda")
+    Xe = torch.empty(L, K + 128, dtype=torch.uint8, device="cuda")
+    s_a = torch.empty(L, dtype=torch.float32, device="cuda")
+    z_a = torch.empty(L, dtype=torch.int32, device="cuda")
+    abi.sgat_quantize_act_asym(X, H.dev(case.mask), H.dev(xf.a_m), H.dev(xf.a_u), hb, xf.d_sh, xf.d_m, xf.d_u, Xq, s_a,
+                               z_a, Xe=Xe)
+    torch.cuda.synchronize()
+    codes, s, z = osg.sgat_quantize_act_asym(case.X, case.mask, xf.a_m, xf.a_u, hb, xf.d_sh, xf.d_m, xf.d_u)
+    nibbles = Xq.cpu().numpy()
+    assert np.array_equal(np.stack([nibbles & 15, nibbles >> 4], -1).reshape(L, K), codes)
+    assert np.array_equal(Xe[:, :K].view(torch.float8_e4m3fn).float().cpu().numpy(), codes.astype(np.float32))
+    assert np.array_equal(s_a.cpu().numpy(), s)
+    assert np.array_equal(z_a.cpu().numpy(), z)
