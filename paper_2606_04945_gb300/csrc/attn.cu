@@ -217,8 +217,8 @@ __device__ __forceinline__ void named_sync_softmax() {
 // channels (128-byte rows) of up to NCH chunks of 128 keys, and the CTAs of
 // one channel group are a cluster. V is read once, into registers; the CTA's
 // channel maxima go to every CTA of the cluster through distributed shared
-// memory, and after one cluster barrier each quantises its own keys, transposes
-// them through shared memory and writes 256-byte runs of Vt. (One CTA per 16
+// memory (once all have started), and after a cluster barrier each quantises its
+// own keys, transposes them through shared memory and writes 256-byte runs of Vt. (One CTA per 16
 // channels reading V twice took 9.1 us at 1024 x 4096 and, with 32 CTAs, 10.7 at
 // 2048 x 512.)
 // Thread (warp w, lane l): channels 8 (l mod 8) .. + 7 of the key pairs 4 w +
@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(VQ_THREADS) attn_vquant_kernel(AttnArgs a, int
     __shared__ float cl_max[VQ_MAX_SPLIT][VQ_CH];          // the channel maxima of the cluster's CTAs
     __shared__ float rcp[VQ_CH];
     __shared__ __align__(16) uint32_t tile[VQ_CH][ATTN_TILE / 2];
+    cluster_started_arrive();          // waited for ahead of the exchange of the maxima
     grid_dependency_wait();            // launched with programmatic serialisation
     grid_launch_dependents();
     const int rank = (int)cluster_ctarank();
@@ -275,14 +276,15 @@ __global__ void __launch_bounds__(VQ_THREADS) attn_vquant_kernel(AttnArgs a, int
         for (int k = 0; k < 8; ++k) red[warp][8 * lane + k] = m[k];
     }
     __syncthreads();
+    cluster_started_wait();      // every CTA runs: its shared memory may be written
     if (tid < VQ_CH) {
         float mm = 0.f;
         #pragma unroll
         for (int w = 0; w < VQ_THREADS / 32; ++w) mm = fmaxf(mm, red[w][tid]);
         for (int c = 0; c < split; ++c)
-            asm volatile("st.shared::cluster.f32 [%0], %1;"
-                         :: "r"(mapa_shared(smem_addr(&cl_max[rank][tid]), (uint32_t)c)), "f"(mm) : "memory");
+            st_shared_cluster_f32(mapa_shared(smem_addr(&cl_max[rank][tid]), (uint32_t)c), mm);
     }
+    __syncwarp();
     cluster_sync();              // nobody touches another CTA's memory after this
     if (tid < VQ_CH) {
         float mm = 0.f;

@@ -464,6 +464,23 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                  ::: "memory");
 }
+// The two halves of a barrier that only says that every CTA of the cluster has
+// started: another CTA's shared memory may be accessed only after that. Arrive
+// as the kernel begins, wait ahead of the first such access; nothing written
+// before the arrival is ordered by it.
+__device__ __forceinline__ void cluster_started_arrive() {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_started_wait() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Stores to the shared memory of any CTA of the cluster (shared::cluster address).
+__device__ __forceinline__ void st_shared_cluster_b32(uint32_t cluster_addr, uint32_t v) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" :: "r"(cluster_addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_shared_cluster_f32(uint32_t cluster_addr, float v) {
+    st_shared_cluster_b32(cluster_addr, __float_as_uint(v));
+}
 // 2-D TMA tile load global -> this CTA's shared memory, completion counted
 // on `bar` (bytes).
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int x, int y,

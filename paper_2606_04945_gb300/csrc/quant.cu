@@ -522,10 +522,6 @@ __device__ __forceinline__ uint32_t e4m3_bytes4(const float* qf) {
     return (uint32_t)h[0] | ((uint32_t)h[1] << 16);
 }
 
-__device__ __forceinline__ void st_shared_cluster_f32(uint32_t cluster_addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" :: "r"(cluster_addr), "f"(v) : "memory");
-}
-
 // Four consecutive elements of a row as loaded, and as float32.
 template <typename T> struct Raw4 { using V = uint2; };
 template <> struct Raw4<float> { using V = float4; };
@@ -567,6 +563,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
     __shared__ __align__(16) float buf[4 * SLICE];
     __shared__ float red[8];              // [0, 4) amax or X_max, [4, 8) -X_min (asym)
     __shared__ float cl_red[2][MAX_SLICES];   // the maxima (and -minima) of the row's slices
+    if (CLUSTER) cluster_started_arrive();    // waited for ahead of the exchange of the maxima
     // launched with programmatic serialisation: the rows of a problem whose
     // caller vouches that the preceding launch neither writes its inputs
     // nor touches its outputs start without waiting for that launch
@@ -731,12 +728,15 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
     if (ASYM) nmin = fmaxf(fmaxf(red[4], red[5]), fmaxf(red[6], red[7]));
     if (CLUSTER) {
         // the row's maximum over the cluster's slices: every CTA writes its
-        // own into all of them, so that after the one barrier nobody reads
-        // another CTA's memory and each may finish by itself
+        // own into all of them, once all have started, so that after the
+        // second barrier nobody reads another CTA's memory and each may finish
+        // by itself
+        cluster_started_wait();
         if ((int)threadIdx.x < ctas_per_row) {
             st_shared_cluster_f32(mapa_shared(smem_addr(&cl_red[0][rank]), threadIdx.x), amax);
             if (ASYM) st_shared_cluster_f32(mapa_shared(smem_addr(&cl_red[1][rank]), threadIdx.x), nmin);
         }
+        __syncwarp();
         cluster_sync();
         for (int c = 0; c < ctas_per_row; ++c) {
             amax = fmaxf(amax, cl_red[0][c]);

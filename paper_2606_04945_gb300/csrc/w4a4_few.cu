@@ -89,9 +89,6 @@ __device__ __forceinline__ void store4(float* p, const float (&y)[4]) {
 __device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.b32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ void st_shared_cluster_b32(uint32_t cluster_addr, uint32_t v) {
-    asm volatile("st.shared::cluster.b32 [%0], %1;" :: "r"(cluster_addr), "r"(v) : "memory");
-}
 
 // blockIdx.x = channel tile * split + part, the cluster being the parts of one
 // tile; blockIdx.y = token tile.
