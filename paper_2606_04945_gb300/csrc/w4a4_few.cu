@@ -26,8 +26,9 @@
 //   warp 5    TMEM allocation, MMA issue (tcgen05 kind::f8f6f4, M 128, N NT);
 //   warps 0-3 accumulator to the parts that own the tokens, their sums,
 //             dequantisation, stores.
-// Every wait is bounded; a CTA that gives up records it in the status word
-// and still takes part in the cluster barriers.
+// Every wait is bounded; a CTA that gives up records it in the status word,
+// takes part in the cluster barriers all the same, stores nothing and leaves
+// only when the tiles it has asked for have landed.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -131,6 +132,7 @@ w4a4_gemm_few_kernel(GemmArgs a, const __grid_constant__ CUtensorMap tmap_w, con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
+    int issued = 0;                                          // TMA warp: K blocks asked for
     float sa_lane = 0.f;                                     // epilogue: scales and bias, read ahead
     bool ok_epi = false;
     float4 sw = make_float4(0.f, 0.f, 0.f, 0.f), bb = sw;
@@ -155,9 +157,11 @@ w4a4_gemm_few_kernel(GemmArgs a, const __grid_constant__ CUtensorMap tmap_w, con
             }
         }
         __syncwarp();
+        issued = pre;
         for (int kc = pre; kc < nk && ok; ++kc) {
             const int s = kc % STAGES;
             ok = mbar_wait_bounded_warp(smem_addr(&sh->empty[s]), (uint32_t)((kc / STAGES) & 1) ^ 1u, abort);
+            if (ok) ++issued;
             if (ok && elect_one()) {
                 const uint32_t st = base + s * STAGE_BYTES, bar = smem_addr(&sh->full[s]);
                 mbar_arrive_expect_tx(bar, STAGE_BYTES);
@@ -253,7 +257,7 @@ w4a4_gemm_few_kernel(GemmArgs a, const __grid_constant__ CUtensorMap tmap_w, con
     // this part's tokens are complete; no part touches another's memory any more
     if (split > 1) cluster_sync();
     else __syncthreads();
-    if (warp < fewk::NUM_EPI_WARPS) {
+    if (warp < fewk::NUM_EPI_WARPS && ok_epi && *abort == 0) {
         TOut* Y = static_cast<TOut*>(a.Y);
         int j = 0;                                           // tokens finished by this warp
         for (int sl = warp; part + sl * split < L; sl += fewk::NUM_EPI_WARPS, ++j) {
@@ -307,6 +311,16 @@ w4a4_gemm_few_kernel(GemmArgs a, const __grid_constant__ CUtensorMap tmap_w, con
     __syncwarp();
     tc_fence_after();
     if (warp == fewk::MMA_WARP) tmem_dealloc(tmem, Tile::TMEM_COLS);
+    if (warp == fewk::TMA_WARP && *abort != 0) {
+        // one of the roles gave up (set before the barrier above), and nobody
+        // has waited for the tiles that the MMA warp did not reach: the CTA must
+        // not give its shared memory back under them (the last use of each
+        // stage, read or not). Out of the way of the epilogue's code: ahead of it
+        // the same lines cost 0.05 us a launch.
+        volatile int never = 0;
+        for (int kc = issued > STAGES ? issued - STAGES : 0; kc < issued; ++kc)
+            if (!mbar_wait_bounded_warp(smem_addr(&sh->full[kc % STAGES]), (uint32_t)((kc / STAGES) & 1), &never)) break;
+    }
 }
 
 bool encode_k_major(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t elem) {
