@@ -331,9 +331,10 @@ size_t sgat_linear_asym_workspace_size(int L, int K);
  * Dense orthogonal basis (the learned P of App. B; W_f = Q_w(P^T W^T)) in
  * place of the block Hadamard transform. The transform X^s P is a 16-bit
  * GEMM: its operands are the scaled rows fl16(fl32(x * a_s)) and P, both
- * float16, accumulated in float32 on the tensor cores, and the result is
- * stored as float16. The gate and the symmetric 4-bit quantiser (hb = 1)
- * then run on it.
+ * float16, accumulated in float32 on the tensor cores (one chain over K for
+ * every batch: a row's codes do not depend on the other rows of the call, nor
+ * on starq_set_gemm_pair_limit), and the result is stored as float16. The gate
+ * and the symmetric 4-bit quantiser (hb = 1) then run on it.
  *
  *   Pt [K][K] float16: the basis transposed (row j holds column j of P),
  *      16-byte aligned. P must be orthogonal: the weight side then uses the
@@ -435,7 +436,8 @@ int w4a4_gemm_grouped(const uint8_t* Xe0, const float* s_a0, const uint8_t* We0,
  * 0 removes the cap. Returns the previous cap (>= 0), or STARQ_ERR_ARG for
  * pairs < 0. The cap is part of the launch, so a CUDA graph captured under
  * it keeps it. Use: a GEMM that runs beside other kernels (two branches of
- * one step) leaves them the remaining SMs; the results do not depend on it.
+ * one step) leaves them the remaining SMs. The results do not depend on it,
+ * but for the rounding of fp16_gemm_ref with few rows (see there).
  */
 int starq_set_gemm_pair_limit(int pairs);
 
@@ -467,7 +469,8 @@ int w4a4_gemm_mma_sync(const uint8_t* Xq, const float* s_a, const uint8_t* Wq, c
  * launcher estimates each shape's time (rounds of tiles over the resident
  * pairs, the weight stream, the exchange of a split K) and takes the cheapest;
  * under a cap on the pairs (starq_set_gemm_pair_limit) always pair tiles. A
- * diagnostic for tests and tuning; the results do not depend on it.
+ * diagnostic for tests and tuning; the results do not depend on it, but for
+ * the rounding of fp16_gemm_ref (see there).
  */
 int starq_last_gemm_tile(void);
 
@@ -477,7 +480,9 @@ int starq_last_gemm_tile(void);
  * unquantised model's linear layer that Sec. 4.4 measures its speed-up
  * against; here it serves only as that denominator (the same tcgen05 kernels
  * as w4a4_gemm, CTA pairs or the few-token one that splits K, kind::f16, no
- * cuBLAS; the order of the float32 sums is the kernel's).
+ * cuBLAS). The order of the float32 sums is the kernel's: with up to 256 rows
+ * and no cap on the pairs K may be summed in up to eight parts, their number
+ * following M, N and K.
  *
  *   A [M][K], B [N][K] row-major, C [M][N] out; all of element type dtype
  *   (F16 or BF16), 16-byte aligned.

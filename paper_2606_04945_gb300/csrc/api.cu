@@ -147,13 +147,17 @@ int check_local(const char* who, cudaStream_t stream, std::initializer_list<cons
 
 // The dense-basis transform of `rows` rows into V (float16): the scaled
 // rows fl16(fl32(x * a_s)) into Xs, then V = Xs P on the 16-bit GEMM
-// (B operand Pt = P^T).
+// (B operand Pt = P^T). V is quantised next, so its float32 sums keep one order
+// for every batch: with the few-token kernel's split of K, which follows L, a
+// token's codes moved with the number of other tokens in the call. (32 x 4096
+// the product alone 9.0 us there and 19.2 here.)
 cudaError_t dense_transform(const void* X, int x_dtype, int rows, int K, const uint8_t* mask, const float* a_m,
                             const float* a_u, const void* Pt, __half* Xs, __half* V, unsigned* st, cudaStream_t s) {
     cudaError_t e = launch_scale_rows_f16(X, x_dtype, rows, K, mask, a_m, a_u, Xs, s);
     if (e != cudaSuccess) return e;
     GemmArgs g{nullptr, nullptr, nullptr, nullptr, nullptr, rows, K, K, V, STARQ_F16, nullptr, st,
                reinterpret_cast<const uint8_t*>(Xs), static_cast<const uint8_t*>(Pt)};
+    g.one_chain = 1;
     return launch_fp16_gemm(g, s);
 }
 

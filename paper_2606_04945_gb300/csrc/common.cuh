@@ -71,6 +71,9 @@ struct GemmArgs {
     // Epilogue silu(gate) * up over weight rows interleaved in groups of 16
     // (Xe + We path, 16-bit Y of [L][N / 2]).
     int swiglu = 0;
+    // 16-bit product: every element is one float32 chain over K whatever L is,
+    // so that a row's result does not depend on the rows beside it.
+    int one_chain = 0;
 };
 cudaError_t launch_w4a4_gemm(const GemmArgs& a, cudaStream_t stream);
 // The same product with Xe and We for few tokens (few_tokens(a, opk)): K split

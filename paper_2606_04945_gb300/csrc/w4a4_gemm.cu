@@ -1609,7 +1609,7 @@ static cudaError_t launch_few_tile(const GemmArgs& a, int opk, cudaStream_t stre
 cudaError_t launch_fp16_gemm(const GemmArgs& a, cudaStream_t stream) {
     if (a.L == 0) return cudaSuccess;
     const int opk = a.y_dtype == STARQ_BF16 ? 2 : 1;
-    if (takes_few(a, opk)) return launch_few_tile(a, opk, stream);
+    if (!a.one_chain && takes_few(a, opk)) return launch_few_tile(a, opk, stream);
     switch (a.y_dtype) {
         case STARQ_F16: return launch_tma_typed<__half, 1>(a, stream);
         case STARQ_BF16: return launch_tma_typed<__nv_bfloat16, 2>(a, stream);
