@@ -513,6 +513,17 @@ __device__ __forceinline__ void quant_pair(float v0, float v1, float r, float& q
     i1 -= 0x4B400000;
 }
 
+// Four codes (ints) -> packed nibbles in the low 16 bits, code k in bits 4k ..
+// 4k + 3. Saturating: where the reciprocal scale or a product is infinite the
+// integer is far out of range, and its low bits alone would be any code.
+__device__ __forceinline__ uint16_t pack_nibbles4(const int* q) {
+    uint32_t w = 0;
+    #pragma unroll
+    for (int k = 2; k >= 0; k -= 2)      // d = c << 8 | sat4(a) << 4 | sat4(b)
+        asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %0;" : "+r"(w) : "r"(q[k + 1]), "r"(q[k]));
+    return (uint16_t)w;
+}
+
 // Four codes (floats) -> their E4M3 bytes (byte k = code k).
 __device__ __forceinline__ uint32_t e4m3_bytes4(const float* qf) {
     uint16_t h[2];
@@ -821,8 +832,7 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
                     prmt(prmt((uint32_t)qi[0], (uint32_t)qi[1], 0x0040u),
                          prmt((uint32_t)qi[2], (uint32_t)qi[3], 0x0040u), 0x5410u);
             else
-                *reinterpret_cast<uint16_t*>(dst + first(g) / 2) =
-                    (uint16_t)((qi[0] & 15) | (qi[1] & 15) << 4 | (qi[2] & 15) << 8 | (qi[3] & 15) << 12);
+                *reinterpret_cast<uint16_t*>(dst + first(g) / 2) = pack_nibbles4(qi);
         }
     }
 }

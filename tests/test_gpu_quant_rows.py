@@ -76,3 +76,28 @@ def test_rows_asym_bitexact(abi, L, K, hb, dtype):
     assert np.array_equal(Xe[:, :K].view(torch.float8_e4m3fn).float().cpu().numpy(), codes.astype(np.float32))
     assert np.array_equal(s_a.cpu().numpy(), s)
     assert np.array_equal(z_a.cpu().numpy(), z)
+
+
+@pytest.mark.parametrize("K,hb", [(1024, 1), (2048, 2048), (4096, 1)])
+def test_rows_nibbles_saturate(abi, K, hb):
+    """Packed codes of rows without a finite reciprocal scale saturate: with
+    amax <= 7 / FLT_MAX the reciprocal 7 / amax is infinite, so every product
+    is +-inf and its code the end of the nibble's range on that side; an
+    infinite element has the reciprocal 0, the product inf * 0 (no number) and
+    the code 7, the row's finite elements 0."""
+    L = 2
+    X = np.zeros((L, K), np.float32)
+    X[0] = np.where(np.arange(K) % 3 == 0, 1e-38, -1e-38) if hb == 1 else 0
+    if hb == 1:
+        X[1] = 1.0
+        X[1, 5] = np.inf
+    else:
+        X[0, 0] = 1e-38                                    # its transform: 1e-38 in every element of the block
+    mask = np.zeros(L, np.uint8)
+    Xq = torch.empty(L, K // 2, dtype=torch.uint8, device="cuda")
+    s_a = torch.empty(L, dtype=torch.float32, device="cuda")
+    abi.sgat_quantize_act(H.dev(X), H.dev(mask), None, None, hb, K, 0, 0, Xq, s_a)
+    codes = H.unpack(Xq)
+    assert np.array_equal(codes[0], np.where(X[0] < 0, -8, 7) if hb == 1 else np.full(K, 7))
+    if hb == 1:
+        assert codes[1, 5] == 7 and not np.any(np.delete(codes[1], 5))
