@@ -893,24 +893,25 @@ cudaError_t launch_stream(const TacArgs& a, cudaStream_t stream) {
 
 template <typename TIn, typename TOut>
 cudaError_t launch_io(const TacArgs& a, cudaStream_t stream) {
-    if constexpr (!std::is_same<TIn, float>::value) {
-        if (a.status != nullptr && (a.g == 64 || a.g == 128)) {
-            // prepared halves and more jobs than one wave of the per-tile
-            // kernel (two CTAs per SM) holds: the streaming kernel
-            const long long jobs = (long long)(a.C / a.g) * ((a.L + TC_TM - 1) / TC_TM);
-            if (a.Mp != nullptr && jobs > 2LL * num_sms())
-                return a.g == 64 ? launch_stream<64, TIn, TOut>(a, stream) : launch_stream<128, TIn, TOut>(a, stream);
-            return a.g == 64 ? launch_tc<64, TIn, TOut>(a, stream) : launch_tc<128, TIn, TOut>(a, stream);
-        }
-    }
     switch (a.g) {
         case 4: return launch_small<4, TIn, TOut>(a, stream);
         case 8: return launch_small<8, TIn, TOut>(a, stream);
         case 16: return launch_small<16, TIn, TOut>(a, stream);
         case 32: return launch_small<32, TIn, TOut>(a, stream);
-        case 64: return launch_g<64, TIn, TOut>(a, stream);
-        case 128: return launch_g<128, TIn, TOut>(a, stream);
+        case 64:
+        case 128: break;
         default: return cudaErrorInvalidValue;
+    }
+    if constexpr (std::is_same<TIn, float>::value) {
+        return a.g == 64 ? launch_g<64, TIn, TOut>(a, stream) : launch_g<128, TIn, TOut>(a, stream);
+    } else {
+        if (a.status == nullptr) return cudaErrorInvalidValue;     // (the tensor-core kernels' bounded waits)
+        // prepared halves and more jobs than one wave of the per-tile
+        // kernel (two CTAs per SM) holds: the streaming kernel
+        const long long jobs = (long long)(a.C / a.g) * ((a.L + TC_TM - 1) / TC_TM);
+        if (a.Mp != nullptr && jobs > 2LL * num_sms())
+            return a.g == 64 ? launch_stream<64, TIn, TOut>(a, stream) : launch_stream<128, TIn, TOut>(a, stream);
+        return a.g == 64 ? launch_tc<64, TIn, TOut>(a, stream) : launch_tc<128, TIn, TOut>(a, stream);
     }
 }
 

@@ -1,6 +1,7 @@
-"""TAC for blocks of up to 32 (CUDA cores, tiles of 128 channels x 128 tokens)
-against float32 sums in the kernel's order (ascending inputs, fused multiply-add,
-then + d): bit for bit, at the edges of its tiles."""
+"""TAC for blocks of up to 32 (CUDA cores, tiles of 128 channels x 64 tokens, 128
+for blocks of 32; a thread takes two tokens half a tile apart) against float32
+sums in the kernel's order (ascending inputs, fused multiply-add, then + d): bit
+for bit but for double roundings of the reference, at the edges of its tiles."""
 
 import numpy as np
 import pytest
@@ -15,7 +16,13 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("g,L,C,zin,zout,with_d", [(4, 1, 8, "f16", "f16", True), (4, 130, 4096, "bf16", "f32", True),
                                                   (8, 127, 136, "f16", "bf16", False), (8, 128, 128, "f32", "f16", True),
                                                   (16, 129, 272, "f16", "f16", True), (16, 300, 2560, "bf16", "bf16", False),
-                                                  (32, 64, 96, "f32", "f32", True), (32, 257, 160, "f16", "f16", True)])
+                                                  (32, 64, 96, "f32", "f32", True), (32, 257, 160, "f16", "f16", True),
+                                                  # one tile of 64 tokens: its halves' edges, its last token, one more
+                                                  (4, 31, 136, "f16", "f16", True), (8, 32, 128, "bf16", "f32", True),
+                                                  (16, 33, 272, "f16", "f16", False), (4, 63, 8, "f32", "f32", True),
+                                                  (8, 64, 264, "f16", "f16", True), (16, 65, 128, "bf16", "bf16", True),
+                                                  (8, 63, 128, "f16", "f16", True), (16, 64, 48, "f16", "f32", True),
+                                                  (4, 65, 128, "f16", "bf16", True)])
 def test_tac_small_blocks(abi, g, L, C, zin, zout, with_d):
     rng = np.random.default_rng(g + L + C)
     Z = rng.standard_normal((L, C)).astype(np.float32)
