@@ -152,9 +152,15 @@ def _p(t):
     return None if t is None else t.data_ptr()
 
 
+# (both private to torch: without them, the public way to the same handle)
+_RAW_STREAM = all(hasattr(torch._C, f) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
+
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
+    if not _RAW_STREAM:
+        return torch.cuda.current_stream().cuda_stream
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 

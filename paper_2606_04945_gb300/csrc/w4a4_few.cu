@@ -352,7 +352,7 @@ FewPlan few_plan(const GemmArgs& a, int opk) {
     p.ctas = tiles * p.rows * p.split;
     const int most = (p.stages + p.split - 1) / p.split;     // stages of the longest part
     const int need = opk == 3 ? (most + fewk::ACC_STAGES - 1) / fewk::ACC_STAGES : 1;
-    p.accs = need <= 1 ? 1 : need <= 2 ? 2 : need;
+    p.accs = need < 1 ? 1 : need;
     return p;
 }
 

@@ -397,3 +397,15 @@ def test_gemm_pair_limit(lib):
         assert lib.set_gemm_pair_limit(0) == 12
     finally:
         lib.set_gemm_pair_limit(prev)
+
+
+def test_current_stream_without_the_private_functions(lib, monkeypatch):
+    """Where torch lacks its private accessors, the current stream's handle
+    comes from the public call."""
+    import types
+
+    import torch
+    monkeypatch.setattr(lib, "_RAW_STREAM", False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=7))
+    assert lib._stream(None) == 7
+    assert lib._stream(types.SimpleNamespace(cuda_stream=9)) == 9
