@@ -29,7 +29,11 @@
 // with weight rows ending in E4M3 values that sum to sum_k q_w, the 4-bit
 // GEMM over K + 128 then gives sum_k (q_a - z) q_w exactly).
 //
-// Work split: a warp owns a chunk of C = 32 E consecutive elements of a row
+// Two kernels. sgat_quant_rows_kernel (further down, with its layouts) takes
+// rows of 1024 features and more, in multiples of 1024 (of 512 with blocks of
+// at most 512). sgat_quant_kernel takes the other shapes:
+//
+// A warp owns a chunk of C = 32 E consecutive elements of a row
 // (C = 1024 when hb >= 1024, else C = 512 holding 512 / hb Hadamard blocks).
 // In layout A lane l holds elements E l .. E l + E - 1, so stages h < E are
 // butterflies between registers of one thread. One transpose through shared
@@ -433,20 +437,20 @@ template <> struct To<float> { static __device__ __forceinline__ float f(float h
 // every address is a per-thread base plus a constant. Only layout 3 and the
 // row maximum need the whole CTA.
 //
-// Bound by instruction issue and shared-memory wavefronts (67% and 74% busy at
-// 8192 x 4096 and seven CTAs per SM), not by HBM. An earlier split (32 consecutive
-// elements per lane first, then two more layouts) staged x and the smoothing
-// vector through shared memory to reach its first layout: 224 wavefronts per
-// 1024 elements instead of 128 (192 with layout 3), and 1141 warp instructions
-// instead of 859 (1349 for the present split with the Hadamard block known
-// only at run time: the branches around the stages keep the register pairs
-// apart). Microseconds back to back, before and now: 8192 x 4096 fp16, hb 4096
-// 43.0, 33.2; 8192 x 3584 bf16, hb 512 39.8, 29.3; 8192 x 18944 245.6, 166;
-// 1024 x 12288 23.5, 17.6; 1024 x 4096 8.3, 6.5; codes of 24576 x 4096 weights
-// 120.5, 92.0; asymmetric 8192 x 4096 47.3, 39.7. Rows shorter than a slice
-// (warps without a chunk leave before the codes), with the idle warps working and
-// now: 8192 x 1024 24.7, 18.6; 8192 x 2048 33.2, 24.4; asymmetric 31.8, 20.9 and
-// 39.5, 27.5.
+// Bound by instruction issue and shared-memory wavefronts (64% and 78% busy at
+// 8192 x 4096), not by HBM. An earlier split (32 consecutive elements per lane
+// first, then two more layouts) staged x and the smoothing vector through shared
+// memory to reach its first layout: 224 wavefronts per 1024 elements instead of
+// 128 (192 with layout 3), and 1141 warp instructions instead of 859, or 789 with
+// FULL (1349 for the present split while the Hadamard block was known only at
+// run time: the branches around the stages keep the register pairs apart).
+// Microseconds back to back, the earlier split and now, one box: 8192 x 4096
+// fp16, hb 4096 42.8, 33.4; 8192 x 3584 bf16, hb 512 39.6, 29.2; 8192 x 18944
+// 244, 168.6; 1024 x 12288 23.4, 17.7; 1024 x 4096 8.2, 6.5; codes of 24576 x 4096
+// weights 120.2, 92.4; asymmetric 8192 x 4096 47.3, 39.7 (another box). Rows
+// shorter than a slice, whose warps without a chunk leave before the codes:
+// 8192 x 1024 22.3, 18.6; 8192 x 2048 29.0, 24.5 (with the idle warps going on,
+// 24.7 and 33.2).
 // Butterflies on pairs of registers use the packed f32x2 add and subtract
 // (each half rounds like the scalar operation).
 // ---------------------------------------------------------------------------
@@ -563,7 +567,7 @@ __device__ __forceinline__ void raw4_to_f(const float4& w, float* f) {
 // 4096: 33.2 against 35.1; 1024 x 12288 17.6, 18.0).
 // CTAs per SM: seven (72 registers); eight (64, no spills for 16-bit inputs)
 // with FULL, and for clustered rows with blocks of 512 (8192 x 18944: 166 us
-// against 176), but not in a single wave (1000 x 3584: 5.7 against 5.3).
+// against 176, both ahead of the barrier that the cluster's start needs), but not in a single wave (1000 x 3584: 5.7 against 5.3).
 template <typename Tin, int HB, bool ASYM, bool CLUSTER, bool G2, bool FULL = false>
 __global__ void __launch_bounds__(128, FULL || (HB == 512 && CLUSTER) ? 8 : 7)
 sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
@@ -840,8 +844,8 @@ sgat_quant_rows_kernel(QuantArgs a0, QuantArgs b, int ctas_per_row) {
 // One launch of the row kernel: a CTA per row (b != nullptr: the rows of b
 // after those of a), or beyond 4096 features a cluster of CTAs per row, one
 // 4096-feature slice each. Blocks of 512 to 4096 are compiled in (8192 x 4096,
-// hb 1024: 30.2 us, against 33.9 with the block at run time; asymmetric, hb 4096,
-// 45.4 and 52.4).
+// hb 1024: 30.2 us, against 33.9 with the block at run time); grouped launches,
+// only 512 and 4096.
 template <typename Tin, bool ASYM, bool CLUSTER, bool G2>
 cudaError_t launch_rows_kind(const QuantArgs& a, const QuantArgs& b, cudaStream_t stream) {
     const int ctas = (a.K + 4095) / 4096;
